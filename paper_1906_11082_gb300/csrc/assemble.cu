@@ -1015,6 +1015,8 @@ int ensure_f32(nm_problem* P, cudaStream_t s) {
     NM_TRY(conv(P->Pn));
     NM_TRY(conv(P->EG));
     NM_TRY(conv(P->EGt));
+    NM_TRY(build_clusters(P->Mr, s));
+    if (P->info.Np > 0) NM_TRY(build_clusters(P->Pn, s));
     return NM_OK;
 }
 

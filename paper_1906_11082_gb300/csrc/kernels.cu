@@ -665,6 +665,7 @@ int launch_kron(int R, int mode, const KronArgs<T>& a, cudaStream_t s) {
     if constexpr (std::is_same<T, float>::value) {
         if (a.tma.ntiles > 0 && R == 3 && mode == KRON_CHEB && a.b == 32 && a.ldx == 32 && !a.chunk && !a.sched)
             return launch_kron_tma(a, s);
+        if (!a.chunk && !a.sched && kron_cluster_ok(R, mode, a)) return launch_kron_cluster(R, mode, a, s);
         if (v4_ok(a) && !a.chunk) {
             if (R == 3) {
                 switch (mode) {
@@ -911,24 +912,24 @@ __global__ void convert_kernel(int64_t rows, int b, const Tin* X, int64_t ldx, T
 
 // w32 = float(W) and the first semi-iteration step x1 = inv_theta D^-1 w32
 // in one pass (the same float expression as dscale_kernel).
-__global__ void convert_x1_kernel(int R, int64_t nodes, int b, const double* W, int64_t ldw, float* w32,
+__global__ void convert_x1_kernel(int R, int64_t nodes, int b, int bv, const double* W, int64_t ldw, float* w32,
                                   float inv_theta, const float* dinv, float* x1) {
     const int64_t total = (int64_t)R * nodes * b;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
          t += (int64_t)gridDim.x * blockDim.x) {
         const int64_t r = t / b;
         const int c = (int)(t - r * b);
-        const float w = (float)W[r * ldw + c];
+        const float w = c < bv ? (float)W[r * ldw + c] : 0.f;
         w32[t] = w;
-        x1[t] = inv_theta * dinv[r / R] * w;
+        if (x1) x1[t] = inv_theta * dinv[r / R] * w;
     }
 }
 
-int launch_convert_x1(int R, int64_t nodes, int b, const double* W, int64_t ldw, float* w32, float inv_theta,
+int launch_convert_x1(int R, int64_t nodes, int b, int bv, const double* W, int64_t ldw, float* w32, float inv_theta,
                       const float* dinv, float* x1, cudaStream_t s) {
     const int64_t total = (int64_t)R * nodes * b;
     if (total == 0) return NM_OK;
-    convert_x1_kernel<<<grid_for(total), kThreads, 0, s>>>(R, nodes, b, W, ldw, w32, inv_theta, dinv, x1);
+    convert_x1_kernel<<<grid_for(total), kThreads, 0, s>>>(R, nodes, b, bv, W, ldw, w32, inv_theta, dinv, x1);
     count_launch();
     NM_CUDA(cudaGetLastError());
     return NM_OK;
@@ -1033,12 +1034,48 @@ int launch_dscale(int R, int64_t nodes, int b, T inv_theta, const T* dinv, const
     return NM_OK;
 }
 
+// N consecutive values at p (N = 4: p is 16-byte aligned).
+template <int N>
+__device__ __forceinline__ void load_n(const float* p, float* v) {
+    if constexpr (N == 4) {
+        const float4 t = *reinterpret_cast<const float4*>(p);
+        v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
+    } else {
+        v[0] = *p;
+    }
+}
+template <int N>
+__device__ __forceinline__ void load_n(const double* p, double* v) {
+    if constexpr (N == 4) {
+        const double2 t = reinterpret_cast<const double2*>(p)[0], u = reinterpret_cast<const double2*>(p)[1];
+        v[0] = t.x, v[1] = t.y, v[2] = u.x, v[3] = u.y;
+    } else {
+        v[0] = *p;
+    }
+}
+template <int N>
+__device__ __forceinline__ void store_n(float* p, const float* v) {
+    if constexpr (N == 4)
+        *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    else
+        *p = v[0];
+}
+template <int N>
+__device__ __forceinline__ void store_n(double* p, const double* v) {
+    if constexpr (N == 4) {
+        reinterpret_cast<double2*>(p)[0] = make_double2(v[0], v[1]);
+        reinterpret_cast<double2*>(p)[1] = make_double2(v[2], v[3]);
+    } else {
+        *p = v[0];
+    }
+}
+
 template <int R, int CPT>
 __global__ void __launch_bounds__(kThreads) resid_mixed_kernel(int64_t nodes, const int* __restrict__ rowptr,
                                                                const int* __restrict__ col,
                                                                const double* __restrict__ val,
                                                                const double* __restrict__ W, int64_t ldw,
-                                                               const float* __restrict__ x, float* r, int b,
+                                                               const float* __restrict__ x, float* r, int b, int bv,
                                                                int tpr_shift) {
     const int tpr = 1 << tpr_shift;
     const int lane = threadIdx.x & (tpr - 1);
@@ -1070,54 +1107,77 @@ __global__ void __launch_bounds__(kThreads) resid_mixed_kernel(int64_t nodes, co
 #pragma unroll
         for (int k = 0; k < R; ++k) {
             const int64_t rr = R * row + k;
-            r[rr * b + c] = (float)(W[rr * ldw + c] - acc[q][k]);
+            r[rr * b + c] = (float)((c < bv ? W[rr * ldw + c] : 0.0) - acc[q][k]);
         }
     }
 }
 
 int launch_resid_mixed(int R, int64_t nodes, const int* rowptr, const int* col, const double* val,
-                       const double* W, int64_t ldw, const float* x32, float* r32, int b, cudaStream_t s) {
+                       const double* W, int64_t ldw, const float* x32, float* r32, int b, int bv, cudaStream_t s) {
     if (b < 1 || b > 64) return fail(NM_EINVAL, "block width must be in 1..64");
     const int shift = tpr_shift_for(b);
     const int cpt = (b + (1 << shift) - 1) >> shift;
     const int64_t grid = (nodes + (kThreads >> shift) - 1) / (kThreads >> shift);
     if (grid == 0) return NM_OK;
     if (R == 3 && cpt == 1)
-        resid_mixed_kernel<3, 1><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, val, W, ldw, x32, r32, b, shift);
+        resid_mixed_kernel<3, 1><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, val, W, ldw, x32, r32, b, bv, shift);
     else if (R == 3)
-        resid_mixed_kernel<3, 2><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, val, W, ldw, x32, r32, b, shift);
+        resid_mixed_kernel<3, 2><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, val, W, ldw, x32, r32, b, bv, shift);
     else if (cpt == 1)
-        resid_mixed_kernel<1, 1><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, val, W, ldw, x32, r32, b, shift);
+        resid_mixed_kernel<1, 1><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, val, W, ldw, x32, r32, b, bv, shift);
     else
-        resid_mixed_kernel<1, 2><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, val, W, ldw, x32, r32, b, shift);
+        resid_mixed_kernel<1, 2><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, val, W, ldw, x32, r32, b, bv, shift);
     count_launch();
     NM_CUDA(cudaGetLastError());
     return NM_OK;
 }
 
-__global__ void combine_kernel(const CombineArgs a) {
-    const int64_t total = a.rows * a.b;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const double sv = (double)a.x32[t] + (double)a.e32[t];
+// N columns per thread (4, or 1 where widths or alignments do not allow the
+// vector accesses): 32-bit index arithmetic, the same operations per element.
+template <int N>
+__global__ void __launch_bounds__(kThreads) combine_kernel(const CombineArgs a) {
+    const unsigned nb = a.b / N, total = (unsigned)a.rows * nb;
+    const int dg = a.deg ? a.deg[0] + 1 : 0;
+    const double* gt = a.gam_tab ? a.gam_tab + (int64_t)dg * a.gam_stride : nullptr;
+    for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
+        const unsigned i = t / nb;
+        const int c = N * (int)(t - i * nb), cg = a.c0 + c;
+        const int64_t ix = (int64_t)i * a.ldx + c, it = (int64_t)i * a.ldt + cg;
+        float x[N], e[N];
+        load_n<N>(a.x32 + ix, x);
+        load_n<N>(a.e32 + ix, e);
+        double v[N];
+#pragma unroll
+        for (int j = 0; j < N; ++j) v[j] = (double)x[j] + (double)e[j];
         if (!a.Tn) {
-            a.out[t] = sv;
+            store_n<N>(a.out + it, v);
             continue;
         }
-        const double tp = a.Tp ? a.Tp[t] : 0.0;
-        const double tn = a.a1 * (sv - a.cshift * a.Tk[t]) - a.a2 * tp;
-        a.Tn[t] = tn;
+        double tk[N], tp[N];
+        load_n<N>(a.Tk + it, tk);
+#pragma unroll
+        for (int j = 0; j < N; ++j) tp[j] = 0.0;
+        if (a.Tp) load_n<N>(a.Tp + it, tp);
+#pragma unroll
+        for (int j = 0; j < N; ++j) v[j] = a.a1 * (v[j] - a.cshift * tk[j]) - a.a2 * tp[j];
+        store_n<N>(a.Tn + it, v);
         if (a.Th) {   // exact float pair of tn for the next double-float K_eff SpMM
-            const float h = __double2float_rn(tn);
-            a.Th[t] = h;
-            a.Tl[t] = __double2float_rn(tn - (double)h);
+            const int64_t ih = (int64_t)i * a.ldh + cg;
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                x[j] = __double2float_rn(v[j]);
+                e[j] = __double2float_rn(v[j] - (double)x[j]);
+            }
+            store_n<N>(a.Th + ih, x);
+            store_n<N>(a.Tl + ih, e);
         }
         if (a.Z) {
-            const int64_t i = t / a.b;
-            const int c = (int)(t - i * a.b);
-            const double gm = a.deg ? a.gam_tab[(int64_t)(a.deg[0] + 1) * a.gam_stride + c / a.gam_group]
-                                    : (a.gam_tab ? a.gam_tab[c / a.gam_group] : a.gam);
-            a.Z[i * a.ldz + c] += gm * tn;
+            const int64_t iz = (int64_t)i * a.ldz + cg;
+            double z[N];
+            load_n<N>(a.Z + iz, z);
+#pragma unroll
+            for (int j = 0; j < N; ++j) z[j] += (gt ? gt[(cg + j) / a.gam_group] : a.gam) * v[j];
+            store_n<N>(a.Z + iz, z);
         }
     }
 }
@@ -1172,65 +1232,15 @@ int launch_inc_int(int* p, cudaStream_t s) {
     return NM_OK;
 }
 
-// The same update two columns per thread (b even, operands 8/16-byte
-// aligned, Z's leading dimension even, rows * b / 2 < 2^30): 32-bit index
-// arithmetic, float2 / double2 accesses, identical arithmetic per element.
-__global__ void combine2_kernel(const CombineArgs a) {
-    const int hb = a.b >> 1;
-    const int total = (int)(a.rows * hb);
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
-        const float2 x = reinterpret_cast<const float2*>(a.x32)[t];
-        const float2 e = reinterpret_cast<const float2*>(a.e32)[t];
-        const double s0 = (double)x.x + (double)e.x, s1 = (double)x.y + (double)e.y;
-        if (!a.Tn) {
-            reinterpret_cast<double2*>(a.out)[t] = make_double2(s0, s1);
-            continue;
-        }
-        const double2 tk = reinterpret_cast<const double2*>(a.Tk)[t];
-        const double2 tp = a.Tp ? reinterpret_cast<const double2*>(a.Tp)[t] : make_double2(0.0, 0.0);
-        const double n0 = a.a1 * (s0 - a.cshift * tk.x) - a.a2 * tp.x;
-        const double n1 = a.a1 * (s1 - a.cshift * tk.y) - a.a2 * tp.y;
-        reinterpret_cast<double2*>(a.Tn)[t] = make_double2(n0, n1);
-        if (a.Th) {
-            const float h0 = __double2float_rn(n0), h1 = __double2float_rn(n1);
-            reinterpret_cast<float2*>(a.Th)[t] = make_float2(h0, h1);
-            reinterpret_cast<float2*>(a.Tl)[t] =
-                make_float2(__double2float_rn(n0 - (double)h0), __double2float_rn(n1 - (double)h1));
-        }
-        if (a.Z) {
-            const int i = t / hb;
-            const int c = 2 * (t - i * hb);
-            double g0, g1;
-            if (a.deg) {
-                const double* gt = a.gam_tab + (int64_t)(a.deg[0] + 1) * a.gam_stride;
-                g0 = gt[c / a.gam_group];
-                g1 = gt[(c + 1) / a.gam_group];
-            } else if (a.gam_tab) {
-                g0 = a.gam_tab[c / a.gam_group];
-                g1 = a.gam_tab[(c + 1) / a.gam_group];
-            } else {
-                g0 = g1 = a.gam;
-            }
-            double2* zp = reinterpret_cast<double2*>(a.Z + (int64_t)i * a.ldz + c);
-            double2 z = *zp;
-            z.x += g0 * n0;
-            z.y += g1 * n1;
-            *zp = z;
-        }
-    }
-}
-
 int launch_combine(const CombineArgs& a, cudaStream_t s) {
     if (a.rows * a.b == 0) return NM_OK;
-    const uintptr_t al16 = (uintptr_t)a.out | (uintptr_t)a.Tk | (uintptr_t)a.Tp | (uintptr_t)a.Tn | (uintptr_t)a.Z;
-    const uintptr_t al8 = (uintptr_t)a.x32 | (uintptr_t)a.e32 | (uintptr_t)a.Th | (uintptr_t)a.Tl;
-    if (a.b % 2 == 0 && (al16 & 15) == 0 && (al8 & 7) == 0 && (a.ldz % 2) == 0 && a.rows * a.b / 2 < (1ll << 30)) {
-        combine2_kernel<<<grid_for(a.rows * a.b / 2), kThreads, 0, s>>>(a);
-        count_launch();
-        NM_CUDA(cudaGetLastError());
-        return NM_OK;
-    }
-    combine_kernel<<<grid_for(a.rows * a.b), kThreads, 0, s>>>(a);
+    if (a.rows * a.b > 0xFFFFFFFFll) return fail(NM_EINVAL, "block too large for the combine");
+    const uintptr_t al = (uintptr_t)a.out | (uintptr_t)a.Tk | (uintptr_t)a.Tp | (uintptr_t)a.Tn | (uintptr_t)a.Z |
+                         (uintptr_t)a.x32 | (uintptr_t)a.e32 | (uintptr_t)a.Th | (uintptr_t)a.Tl;
+    if (((a.b | a.c0) & 3) == 0 && ((a.ldx | a.ldh) & 3) == 0 && ((a.ldt | a.ldz) & 1) == 0 && (al & 15) == 0)
+        combine_kernel<4><<<grid_for(a.rows * a.b / 4), kThreads, 0, s>>>(a);
+    else
+        combine_kernel<1><<<grid_for(a.rows * a.b), kThreads, 0, s>>>(a);
     count_launch();
     NM_CUDA(cudaGetLastError());
     return NM_OK;
@@ -1253,13 +1263,13 @@ __device__ __forceinline__ void df_fma(float& sh, float& sl, float ah, float al,
     sl = __fadd_rn(lo, -__fadd_rn(sh, -s));
 }
 
-__global__ void split_kernel(int64_t rows, int b, const double* X, int64_t ldx, float* Xh, float* Xl) {
-    const int64_t total = rows * b;
+__global__ void split_kernel(int64_t rows, int b, int ldh, const double* X, int64_t ldx, float* Xh, float* Xl) {
+    const int64_t total = rows * ldh;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
          t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = t / b;
-        const int c = (int)(t - i * b);
-        const double x = X[i * ldx + c];
+        const int64_t i = t / ldh;
+        const int c = (int)(t - i * ldh);
+        const double x = c < b ? X[i * ldx + c] : 0.0;
         const float h = __double2float_rn(x);
         Xh[t] = h;
         Xl[t] = __double2float_rn(x - (double)h);
@@ -1286,7 +1296,7 @@ __global__ void __launch_bounds__(kThreads) bsr33_df_kernel(const Bsr33DfArgs a,
             kh[t] = __ldg(a.vh + 9 * (int64_t)e + t);
             kl[t] = __ldg(a.vl + 9 * (int64_t)e + t);
         }
-        const int64_t base = 3 * j * a.b;
+        const int64_t base = 3 * j * a.ldx;
 #pragma unroll
         for (int q = 0; q < CPT; ++q) {
             const int c = lane + q * tpr;
@@ -1294,8 +1304,8 @@ __global__ void __launch_bounds__(kThreads) bsr33_df_kernel(const Bsr33DfArgs a,
                 float xh[3], xl[3];
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
-                    xh[k] = __ldg(a.Xh + base + k * a.b + c);
-                    xl[k] = __ldg(a.Xl + base + k * a.b + c);
+                    xh[k] = __ldg(a.Xh + base + k * a.ldx + c);
+                    xl[k] = __ldg(a.Xl + base + k * a.ldx + c);
                 }
 #pragma unroll
                 for (int m = 0; m < 3; ++m)
@@ -1330,7 +1340,7 @@ __global__ void __launch_bounds__(kThreads) resid_df_kernel(int64_t nodes, const
                                                             const int* __restrict__ col, const float* __restrict__ vh,
                                                             const float* __restrict__ vl, const double* __restrict__ W,
                                                             int64_t ldw, const float* __restrict__ x, float* r, int b,
-                                                            int tpr_shift) {
+                                                            int bv, int tpr_shift) {
     const int tpr = 1 << tpr_shift;
     const int lane = threadIdx.x & (tpr - 1);
     const int64_t row = (int64_t)blockIdx.x * (kThreads >> tpr_shift) + (threadIdx.x >> tpr_shift);
@@ -1361,7 +1371,7 @@ __global__ void __launch_bounds__(kThreads) resid_df_kernel(int64_t nodes, const
 #pragma unroll
         for (int k = 0; k < R; ++k) {
             const int64_t rr = R * row + k;
-            r[rr * b + c] = (float)((W[rr * ldw + c] - (double)sh[q][k]) - (double)sl[q][k]);
+            r[rr * b + c] = (float)(((c < bv ? W[rr * ldw + c] : 0.0) - (double)sh[q][k]) - (double)sl[q][k]);
         }
     }
 }
@@ -1522,9 +1532,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT) resid_df_v4_kernel(int64_t node
     }
 }
 
-int launch_split(int64_t rows, int b, const double* X, int64_t ldx, float* Xh, float* Xl, cudaStream_t s) {
+int launch_split(int64_t rows, int b, int ldh, const double* X, int64_t ldx, float* Xh, float* Xl, cudaStream_t s) {
     if (rows * b == 0) return NM_OK;
-    split_kernel<<<grid_for(rows * b), kThreads, 0, s>>>(rows, b, X, ldx, Xh, Xl);
+    split_kernel<<<grid_for(rows * ldh), kThreads, 0, s>>>(rows, b, ldh, X, ldx, Xh, Xl);
     count_launch();
     NM_CUDA(cudaGetLastError());
     return NM_OK;
@@ -1532,7 +1542,7 @@ int launch_split(int64_t rows, int b, const double* X, int64_t ldx, float* Xh, f
 
 int launch_bsr33_df(const Bsr33DfArgs& a, cudaStream_t s) {
     if (a.b < 1 || a.b > 64) return fail(NM_EINVAL, "block width must be in 1..64");
-    if (a.vec && a.b == 32 && (((uintptr_t)a.Xh | (uintptr_t)a.Xl) & 15) == 0) {
+    if (a.vec && a.b == 32 && a.ldx == 32 && (((uintptr_t)a.Xh | (uintptr_t)a.Xl) & 15) == 0) {
         const int nt = a.nt;
         const int64_t grid = (a.nrows + nt / 32 - 1) / (nt / 32);
         if (grid == 0) return NM_OK;
@@ -1560,10 +1570,10 @@ int launch_bsr33_df(const Bsr33DfArgs& a, cudaStream_t s) {
 }
 
 int launch_resid_df(int R, int64_t nodes, const int* rowptr, const int* col, const float* vh, const float* vl,
-                    const double* W, int64_t ldw, const float* x32, float* r32, int b, cudaStream_t s, int vec,
+                    const double* W, int64_t ldw, const float* x32, float* r32, int b, int bv, cudaStream_t s, int vec,
                     int nt, const float* dinv, float inv_theta, float* x1) {
     if (b < 1 || b > 64) return fail(NM_EINVAL, "block width must be in 1..64");
-    if (vec && b == 32 && (((uintptr_t)x32 | (uintptr_t)r32 | (uintptr_t)x1) & 15) == 0) {
+    if (vec && b == 32 && bv == 32 && (((uintptr_t)x32 | (uintptr_t)r32 | (uintptr_t)x1) & 15) == 0) {
         if (nt != 32 && nt != 64 && nt != 128) nt = 256;
         const int64_t grid = (nodes + nt / 32 - 1) / (nt / 32);
         if (grid == 0) return NM_OK;
@@ -1595,13 +1605,13 @@ int launch_resid_df(int R, int64_t nodes, const int* rowptr, const int* col, con
     const int64_t grid = (nodes + (kThreads >> shift) - 1) / (kThreads >> shift);
     if (grid == 0) return NM_OK;
     if (R == 3 && cpt == 1)
-        resid_df_kernel<3, 1><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, vh, vl, W, ldw, x32, r32, b, shift);
+        resid_df_kernel<3, 1><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, vh, vl, W, ldw, x32, r32, b, bv, shift);
     else if (R == 3)
-        resid_df_kernel<3, 2><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, vh, vl, W, ldw, x32, r32, b, shift);
+        resid_df_kernel<3, 2><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, vh, vl, W, ldw, x32, r32, b, bv, shift);
     else if (cpt == 1)
-        resid_df_kernel<1, 1><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, vh, vl, W, ldw, x32, r32, b, shift);
+        resid_df_kernel<1, 1><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, vh, vl, W, ldw, x32, r32, b, bv, shift);
     else
-        resid_df_kernel<1, 2><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, vh, vl, W, ldw, x32, r32, b, shift);
+        resid_df_kernel<1, 2><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, vh, vl, W, ldw, x32, r32, b, bv, shift);
     count_launch();
     NM_CUDA(cudaGetLastError());
     if (x1) return launch_dscale<float>(R, nodes, b, inv_theta, dinv, r32, b, x1, b, s);

@@ -35,6 +35,19 @@ struct TmaTiles {
     int* err = nullptr;
 };
 
+// Clusters of four rows of a scalar CSR matrix (kron_cluster.cu): cluster c
+// owns rows[c] (-1: none) and the entries ptr[c] .. ptr[c + 1), a multiple of
+// six; entry e is a distinct column of the four rows and their four values
+// (zero where a row does not store it, and in the padding).
+struct Clusters {
+    int n = 0;
+    int sms = 0;   // SMs of the device that holds them
+    const int* ptr = nullptr;
+    const int* col = nullptr;
+    const float4* val = nullptr;
+    const int4* rows = nullptr;
+};
+
 // Y (or the Chebyshev / filter epilogue) from the scalar CSR matrix A
 // applied as A (x) I_R to row-major blocks of b columns. A node row i owns
 // the R consecutive rows R*i .. R*i+R-1 of every block.
@@ -83,7 +96,20 @@ struct KronArgs {
     int vec_threads_p = 128; // the same for R = 1
     // bulk-copy staged tiles (R = 3, float, b = ldx = 32, CHEB): ntiles > 0 selects mass_tma.cu
     TmaTiles tma;
+    Clusters cl;
 };
+
+// Semi-iteration (CHEB; R = 3 also CHEB_FILT) on clusters of four rows:
+// widths that are multiples of four, 16-byte aligned operands.
+bool kron_cluster_ok(int R, int mode, const KronArgs<float>& a);
+int launch_kron_cluster(int R, int mode, const KronArgs<float>& a, cudaStream_t s);
+// Column groups the clusters are run in: b columns as ng groups of bg (a
+// multiple of four, at most 32; the last group's padding holds zeros).
+inline void cluster_groups(int b, int* ng, int* bg) {
+    const int lanes = (b + 3) / 4;
+    *ng = (lanes + 7) / 8;
+    *bg = 4 * ((lanes + *ng - 1) / *ng);
+}
 
 // The staged float mass step (one Chebyshev semi-iteration step of
 // M_rho (x) I_3 on 32 columns): persistent CTAs, one producer warp filling
@@ -147,14 +173,21 @@ int launch_dscale(int R, int64_t nodes, int b, T inv_theta, const T* dinv, const
 
 // r32 = float(W - (A (x) I_R) x32) with double matrix values and double
 // sums over the float iterate (the refinement residual of a mixed solve).
+// x32, r32 dense (ld b); W holds the first bv of the b columns (the others
+// count as zero).
 int launch_resid_mixed(int R, int64_t nodes, const int* rowptr, const int* col, const double* val,
-                       const double* W, int64_t ldw, const float* x32, float* r32, int b, cudaStream_t s);
+                       const double* W, int64_t ldw, const float* x32, float* r32, int b, int bv, cudaStream_t s);
 
 // S = double(x32) + double(e32); with Tn != nullptr the outer filter update
-// Tn = a1 (S - c Tk) - a2 Tp, Z += gam Tn, else out = S.
+// Tn = a1 (S - c Tk) - a2 Tp, Z += gam Tn, else out = S. The b columns are
+// the columns c0 .. c0 + b - 1 of the double blocks (out, Tk, Tp, Tn with
+// leading dimension ldt, Z with ldz) and of the float pair (ldh), and the
+// first b of the rows of x32 and e32 (ldx).
 struct CombineArgs {
     int64_t rows = 0;
     int b = 0;
+    int c0 = 0;
+    int64_t ldx = 0, ldt = 0, ldh = 0;
     const float* x32 = nullptr;
     const float* e32 = nullptr;
     double* out = nullptr;
@@ -166,7 +199,7 @@ struct CombineArgs {
     double a1 = 0, cshift = 0, a2 = 0, gam = 0;
     const double* gam_tab = nullptr;   // per column group gamma (overrides gam)
     int gam_group = 1;
-    float* Th = nullptr;   // optional exact float pair (hi, lo) of Tn, dense
+    float* Th = nullptr;   // optional exact float pair (hi, lo) of Tn
     float* Tl = nullptr;
     // graph replay: gamma = gam_tab[(deg[0] + 1) * gam_stride + c / gam_group]
     // with the degree read from device memory (overrides gam and gam_tab's
@@ -186,10 +219,11 @@ int launch_bsr31_add(int nrows, const int* rowptr, const int* col, const double*
 
 // Double-float forms (value = hi + lo, two floats, ~2^-48 relative): the
 // K_eff SpMM and the refinement residual on the float units.
-// Split a double block into exact float pairs (hi = fl(x), lo = fl(x - hi)).
-int launch_split(int64_t rows, int b, const double* X, int64_t ldx, float* Xh, float* Xl, cudaStream_t s);
+// Split a double block into exact float pairs (hi = fl(x), lo = fl(x - hi)),
+// ldh columns wide, those from b on zero.
+int launch_split(int64_t rows, int b, int ldh, const double* X, int64_t ldx, float* Xh, float* Xl, cudaStream_t s);
 // W = A X + E S with A's 3x3 blocks as (hi, lo) floats and X as (hi, lo)
-// float blocks (ld b), double-float sums; the optional E S part in double.
+// float blocks (ld ldx), double-float sums; the optional E S part in double.
 struct Bsr33DfArgs {
     int nrows = 0;
     const int* rowptr = nullptr;
@@ -199,6 +233,7 @@ struct Bsr33DfArgs {
     const float* Xh = nullptr;
     const float* Xl = nullptr;
     int b = 0;
+    int ldx = 0;
     const int* e_rowptr = nullptr;
     const int* e_col = nullptr;
     const double* e_val = nullptr;
@@ -211,15 +246,17 @@ struct Bsr33DfArgs {
 };
 int launch_bsr33_df(const Bsr33DfArgs& a, cudaStream_t s);
 // r32 = float(W - (A (x) I_R) x32) with A as (hi, lo) floats, double-float
-// sums; x32 and r32 dense (ld b). vec: lane-group kernel when b = 32.
+// sums; x32 and r32 dense (ld b); W holds the first bv of the b columns.
+// vec: lane-group kernel when b = bv = 32.
 int launch_resid_df(int R, int64_t nodes, const int* rowptr, const int* col, const float* vh, const float* vl,
-                    const double* W, int64_t ldw, const float* x32, float* r32, int b, cudaStream_t s,
+                    const double* W, int64_t ldw, const float* x32, float* r32, int b, int bv, cudaStream_t s,
                     int vec = 1, int nt = 256, const float* dinv = nullptr, float inv_theta = 0.f,
                     float* x1 = nullptr);
 // With x1 != nullptr also writes the first semi-iteration step on r32,
 // x1 = inv_theta D^-1 r32 (dinv per node, ld b).
-// w32 = float(W) and x1 = inv_theta D^-1 w32 in one pass (w32, x1 dense).
-int launch_convert_x1(int R, int64_t nodes, int b, const double* W, int64_t ldw, float* w32, float inv_theta,
+// w32 = float(W) and, with x1 != nullptr, x1 = inv_theta D^-1 w32 in one pass
+// (w32, x1 dense, b wide; W holds the first bv columns, the others are zero).
+int launch_convert_x1(int R, int64_t nodes, int b, int bv, const double* W, int64_t ldw, float* w32, float inv_theta,
                       const float* dinv, float* x1, cudaStream_t s);
 
 // Y[i, c] = alpha * X[i, c] (rows x b, row-major with leading dims).

@@ -93,10 +93,16 @@ struct DevCSR {
     // built on first use: state 0 not built, 1 built, -1 not eligible
     int tma_state = 0;
     TmaTiles tma;
+    // clusters of four rows for the float semi-iteration (kron_cluster.cu),
+    // built on first use: state 0 not built, 1 built, -1 not eligible
+    int cl_state = 0;
+    Clusters cl;
+    DevBuf cl_ptr, cl_col, cl_val, cl_rows;
     DevBuf tma_desc, tma_ucol, tma_lcol, tma_vals, tma_rowptr, tma_dinv, tma_ldiag, tma_err;
 };
 
 int build_tma_tiles(DevCSR& A, cudaStream_t s);
+int build_clusters(DevCSR& A, cudaStream_t s);
 
 struct Workspace {
     DevBuf buf;      // filter recurrence scratch

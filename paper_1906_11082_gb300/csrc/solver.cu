@@ -109,6 +109,17 @@ static void set_tiles(KronArgs<T>& a, const DevCSR& A) {
     a.tile_kernel = A.tile_kernel;
 }
 
+// Float steps run on the four-row clusters unless an option asks for another
+// schedule of the rows.
+static bool use_clusters(const DevCSR& A, const nm_problem* P) {
+    return A.cl_state == 1 && P->use_vec && !P->use_chunk && !P->use_sched;
+}
+
+template <typename T>
+static void set_clusters(KronArgs<T>& a, const DevCSR& A, const nm_problem* P) {
+    if (sizeof(T) == sizeof(float) && use_clusters(A, P)) a.cl = A.cl;
+}
+
 struct ChebCoef {
     double inv_theta, four_sig2;
     ChebCoef(double lo, double hi) {
@@ -178,6 +189,7 @@ static int schur_pressure(const Mats<T>& m, const T* X, int64_t ldx, int b, int 
         a.dinv = m.dP;
         set_tiles(a, *m.Pcsr);
         set_sched(a, m.P);
+        set_clusters(a, *m.Pcsr, m.P);
         a.b = b;
         a.X = buf[(j - 1) & 1];
         a.ldx = b;
@@ -271,6 +283,7 @@ static int mass_steps(const Mats<T>& m, int b, int k_M, double lo, double hi, co
         a.dinv = m.dM;
         set_tiles(a, *m.Mcsr);
         set_sched(a, m.P);
+        set_clusters(a, *m.Mcsr, m.P);
         a.b = b;
         a.X = buf[(j - 1) & 1];
         a.ldx = b;
@@ -366,34 +379,45 @@ static int filter_core(nm_problem* P, const nm_filter* f, const T* Y, int64_t ld
 
 // ------------------------------------------------------------------ mixed precision
 // Scratch: doubles TA, TB, W (n x b), S64, Q64 (Np x b); floats w32, xa, xb,
-// xs, es (n x b; the pressure solve reuses their first Np x b entries).
+// xs, es (n x bg; the pressure solve reuses their first Np x bg entries) and
+// Th, Tl (n x bp). The float solves run on ng column groups of bg columns,
+// one group after the other: their steps then work on dense blocks of at
+// most 32 columns, whose set stays nearer to the L2 cache than the whole
+// block's. bp = ng bg; the padding columns of the last group hold zeros.
 struct MixScratch {
     double *TA, *TB, *W, *S64, *Q64;
     float *w32, *xa, *xb, *xs, *es;
     float *Th, *Tl;   // double-float split of the block K_eff is applied to
+    int ng = 1, bg = 0, bp = 0;
 };
 
 static int get_mix_scratch(nm_problem* P, int b, MixScratch& S) {
     const int64_t n = P->info.n, Np = P->info.Np;
-    const size_t need = (size_t)(3 * n + 2 * Np) * b * sizeof(double) + (size_t)7 * n * b * sizeof(float);
+    S.ng = 1;
+    S.bg = b;
+    if (use_clusters(P->Mr, P) && !(b == 32 && P->use_tma)) cluster_groups(b, &S.ng, &S.bg);
+    S.bp = S.ng * S.bg;
+    // 16-byte aligned parts
+    const int64_t nd = (n * b + 1) / 2 * 2, pd = (Np * b + 1) / 2 * 2, ng = (n * S.bg + 3) / 4 * 4, np = (n * S.bp + 3) / 4 * 4;
+    const size_t need = (size_t)(3 * nd + 2 * pd) * sizeof(double) + (size_t)(5 * ng + 2 * np) * sizeof(float);
     if (P->ws.bytes < need) {
         P->ws.buf.release();
         NM_TRY(P->ws.buf.alloc(need));
         P->ws.bytes = need;
     }
     double* d = P->ws.buf.as<double>();
-    S.TA = d; d += n * b;
-    S.TB = d; d += n * b;
-    S.W = d; d += n * b;
-    S.S64 = d; d += Np * b;
-    S.Q64 = d; d += Np * b;
+    S.TA = d; d += nd;
+    S.TB = d; d += nd;
+    S.W = d; d += nd;
+    S.S64 = d; d += pd;
+    S.Q64 = d; d += pd;
     float* f = reinterpret_cast<float*>(d);
-    S.w32 = f; f += n * b;
-    S.xa = f; f += n * b;
-    S.xb = f; f += n * b;
-    S.xs = f; f += n * b;
-    S.es = f; f += n * b;
-    S.Th = f; f += n * b;
+    S.w32 = f; f += ng;
+    S.xa = f; f += ng;
+    S.xb = f; f += ng;
+    S.xs = f; f += ng;
+    S.es = f; f += ng;
+    S.Th = f; f += np;
     S.Tl = f;
     return NM_OK;
 }
@@ -435,38 +459,57 @@ static int cheb32(nm_problem* P, const DevCSR& A, int R, int b, int k, double lo
         a.om = (float)om;
         a.inv_theta = (float)cc.inv_theta;
         if (R == 3 && b == 32 && P->use_tma && A.tma_state == 1) a.tma = A.tma;
+        set_clusters(a, A, P);
         NM_TRY(launch_kron<float>(R, KRON_CHEB, a, s));
     }
     if (R == 3) NM_TRY(prof_end(P, s, 2, ev, k - 1));
     return NM_OK;
 }
 
-// Refined solve: x = P32 w, r = w - A x (double), e = P32 r; leaves x in
-// S.xs and e in S.es (the caller combines them).
-static int mixed_solve(nm_problem* P, const DevCSR& A, int R, int b, int k, const double* W, int64_t ldw,
+// Refined solve of one column group: x = P32 w, r = w - A x (double), e =
+// P32 r; leaves x in S.xs and e in S.es (the caller combines them). W points
+// at the group's first column; bv of its S.bg columns exist.
+static int mixed_solve(nm_problem* P, const DevCSR& A, int R, int bv, int k, const double* W, int64_t ldw,
                        const MixScratch& S, bool df, cudaStream_t s) {
+    const int b = S.bg;
     const int64_t rows = R * A.nrows;
     const ChebCoef cc(kMassLo, kMassHi);
     const float it = (float)cc.inv_theta;
     // k >= 2: the float conversion of W and the double-float residual also
     // write the first semi-iteration step, so cheb32 starts at step 2
     const bool fuse = k >= 2;
-    if (fuse)
-        NM_TRY(launch_convert_x1(R, A.nrows, b, W, ldw, S.w32, it, A.dinv32.as<float>(), S.xa, s));
-    else
-        NM_TRY((launch_convert<double, float>(rows, b, W, ldw, S.w32, b, s)));
+    NM_TRY(launch_convert_x1(R, A.nrows, b, bv, W, ldw, S.w32, it, A.dinv32.as<float>(), fuse ? S.xa : nullptr, s));
     NM_TRY(cheb32(P, A, R, b, k, kMassLo, kMassHi, S.w32, S.xa, S.xb, S.xs, s, fuse));
     bool x1 = false;
     if (df) {
         NM_TRY(launch_resid_df(R, A.nrows, A.rowptr.as<int>(), A.col.as<int>(), A.val32.as<float>(),
-                               A.vlo32.as<float>(), W, ldw, S.xs, S.w32, b, s, P->use_vec, P->df_threads,
+                               A.vlo32.as<float>(), W, ldw, S.xs, S.w32, b, bv, s, P->use_vec, P->df_threads,
                                A.dinv32.as<float>(), it, fuse ? S.xa : nullptr));
         x1 = fuse;
     } else {
         NM_TRY(launch_resid_mixed(R, A.nrows, A.rowptr.as<int>(), A.col.as<int>(), A.val.as<double>(), W, ldw,
-                                  S.xs, S.w32, b, s));
+                                  S.xs, S.w32, b, bv, s));
     }
     return cheb32(P, A, R, b, k, kMassLo, kMassHi, S.w32, S.xa, S.xb, S.es, s, x1);
+}
+
+// The same for every column group of a block, each followed by its combine:
+// c holds the combine's operands for the whole block (b columns).
+static int mixed_solve_combine(nm_problem* P, const DevCSR& A, int R, int b, int k, const double* W, int64_t ldw,
+                               const MixScratch& S, CombineArgs c, cudaStream_t s) {
+    c.rows = R * A.nrows;
+    c.x32 = S.xs;
+    c.e32 = S.es;
+    c.ldx = S.bg;
+    c.ldt = b;
+    c.ldh = S.bp;
+    for (int g = 0; g < S.ng; ++g) {
+        c.c0 = g * S.bg;
+        c.b = std::min(S.bg, b - c.c0);
+        NM_TRY(mixed_solve(P, A, R, c.b, k, W + c.c0, ldw, S, P->use_df != 0, s));
+        NM_TRY(launch_combine(c, s));
+    }
+    return NM_OK;
 }
 
 // W = K_eff X in double with the pressure inverse by a refined solve.
@@ -485,7 +528,7 @@ static int apply_K_mixed_core(nm_problem* P, const double* X, int64_t ldx, doubl
     Mats<double> m = mats<double>(P);
     const bool df = P->use_df != 0;
     // pre_split: S.Th / S.Tl already hold the exact float pair of X
-    if (df && !pre_split) NM_TRY(launch_split(P->info.n, b, X, ldx, S.Th, S.Tl, s));
+    if (df && !pre_split) NM_TRY(launch_split(P->info.n, b, S.bp, X, ldx, S.Th, S.Tl, s));
     Bsr33Args<double> a;
     a.nrows = (int)m.Nu;
     a.rowptr = m.u_rp;
@@ -525,14 +568,9 @@ static int apply_K_mixed_core(nm_problem* P, const double* X, int64_t ldx, doubl
         q.Q = S.Q64;
         q.ldq = b;
         NM_TRY(launch_bsr13<double>(q, ps));
-        NM_TRY(mixed_solve(P, P->Pn, 1, b, k_P, S.Q64, b, S, P->use_df != 0, ps));
         CombineArgs c;
-        c.rows = m.Np;
-        c.b = b;
-        c.x32 = S.xs;
-        c.e32 = S.es;
         c.out = S.S64;
-        NM_TRY(launch_combine(c, ps));
+        NM_TRY(mixed_solve_combine(P, P->Pn, 1, b, k_P, S.Q64, b, S, c, ps));
         if (!split_e) {
             a.e_rowptr = m.e_rp;
             a.e_col = m.e_col;
@@ -555,6 +593,7 @@ static int apply_K_mixed_core(nm_problem* P, const double* X, int64_t ldx, doubl
             f.Xh = S.Th;
             f.Xl = S.Tl;
             f.b = b;
+            f.ldx = S.bp;
             f.W = W;
             f.ldw = ldw;
             f.vec = P->use_vec;
@@ -574,6 +613,7 @@ static int apply_K_mixed_core(nm_problem* P, const double* X, int64_t ldx, doubl
     f.Xh = S.Th;
     f.Xl = S.Tl;
     f.b = b;
+    f.ldx = S.bp;
     f.e_rowptr = a.e_rowptr;
     f.e_col = a.e_col;
     f.e_val = a.e_val;
@@ -608,7 +648,14 @@ static int filter_apply_mixed(nm_problem* P, const nm_filter* f, const double* Y
     }
     if (d == 0) return NM_OK;
     NM_TRY(launch_scale_copy<double>(n, b, 1.0, Y, ldy, S.TA, b, s));
-    const int64_t kl = 1 + (P->info.Np > 0 ? 2 * f->k_P + 4 : 0);
+    // launches of one K_eff product and of one mass solve with its combine
+    const int64_t per_k = 2 * (f->k_M - 1) + 3, kl = 1 + (P->info.Np > 0 ? 1 + S.ng * (2 * (f->k_P - 1) + 3) : 0);
+    // the padding columns of the split block stay zero: the combines write
+    // the block's own columns only
+    if (P->use_df && S.bp > b && d > 1) {
+        NM_CUDA(cudaMemsetAsync(S.Th, 0, (size_t)n * S.bp * sizeof(float), s));
+        NM_CUDA(cudaMemsetAsync(S.Tl, 0, (size_t)n * S.bp * sizeof(float), s));
+    }
     // One degree k of the recurrence (T_k in cur, T_{k-1} in prev; T_{k+1}
     // overwrites prev). With dev_gam the combine takes gamma_{k+1} from the
     // device table at the device-side degree counter (graph replay).
@@ -619,12 +666,7 @@ static int filter_apply_mixed(nm_problem* P, const nm_filter* f, const double* Y
         NM_TRY(apply_K_mixed(P, cur, b, S.W, b, b, f->k_P, S, s, k > 0 && P->use_df));
         NM_TRY(prof_end(P, s, 1, e0, kl));
         NM_TRY(prof_begin(P, s, &e1));
-        NM_TRY(mixed_solve(P, P->Mr, 3, b, f->k_M, S.W, b, S, P->use_df != 0, s));
         CombineArgs c;
-        c.rows = n;
-        c.b = b;
-        c.x32 = S.xs;
-        c.e32 = S.es;
         c.Tk = cur;
         c.Tp = k == 0 ? nullptr : prev;
         c.Tn = prev;
@@ -649,8 +691,8 @@ static int filter_apply_mixed(nm_problem* P, const nm_filter* f, const double* Y
             c.Th = S.Th;
             c.Tl = S.Tl;
         }
-        NM_TRY(launch_combine(c, s));
-        NM_TRY(prof_end(P, s, 0, e1, 2 * f->k_M + 3));
+        NM_TRY(mixed_solve_combine(P, P->Mr, 3, b, f->k_M, S.W, b, S, c, s));
+        NM_TRY(prof_end(P, s, 0, e1, S.ng * per_k));
         return NM_OK;
     };
     const bool graphs = P->use_graphs && !P->profile && !P->overlap && s != nullptr && d >= 3;
@@ -750,14 +792,9 @@ int solve_M_mixed_pub(nm_problem* P, int k_M, const double* W, int64_t ldw, doub
     if (b == 32 && P->use_tma) NM_TRY(build_tma_tiles(P->Mr, s));
     MixScratch S;
     NM_TRY(get_mix_scratch(P, b, S));
-    NM_TRY(mixed_solve(P, P->Mr, 3, b, k_M, W, ldw, S, P->use_df != 0, s));
     CombineArgs c;
-    c.rows = P->info.n;
-    c.b = b;
-    c.x32 = S.xs;
-    c.e32 = S.es;
     c.out = S.W;
-    NM_TRY(launch_combine(c, s));
+    NM_TRY(mixed_solve_combine(P, P->Mr, 3, b, k_M, W, ldw, S, c, s));
     return launch_scale_copy<double>(P->info.n, b, 1.0, S.W, b, X, ldx, s);
 }
 
