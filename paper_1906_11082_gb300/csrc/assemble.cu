@@ -791,6 +791,7 @@ int assemble(nm_ctx* ctx, const nm_mesh* mesh, const nm_model* mdl, nm_problem* 
     std::vector<int32_t> rp2(rp), cl2(cl);
     NM_TRY(upload_pattern(P->AG, Nu, Nu, 3, 3, std::move(rp), std::move(cl)));
     NM_TRY(upload_pattern(P->Mr, Nu, Nu, 1, 1, std::move(rp2), std::move(cl2)));
+    NM_TRY(build_row_desc(P->Mr));   // A_G has the same pattern
 
     std::vector<int64_t> ftets;
     std::vector<int32_t> ftu, ftp;   // fluid tets: u-nodes and p-nodes
@@ -814,6 +815,7 @@ int assemble(nm_ctx* ctx, const nm_mesh* mesh, const nm_model* mdl, nm_problem* 
         NM_TRY(build_pattern(Np, {gpp}, a, b));
         scatter_positions(a, b, gpp, posP);
         NM_TRY(upload_pattern(P->Pn, Np, Np, 1, 1, std::move(a), std::move(b)));
+        NM_TRY(build_row_desc(P->Pn));
         std::vector<int32_t> c, d;
         NM_TRY(build_pattern(Nu, {gup, gfup}, c, d));
         scatter_positions(c, d, gup, posE);
@@ -824,6 +826,7 @@ int assemble(nm_ctx* ctx, const nm_mesh* mesh, const nm_model* mdl, nm_problem* 
         scatter_positions(e, f, gpu, posEt);
         if (nfs) scatter_positions(e, f, gfpu, posFEt);
         NM_TRY(upload_pattern(P->EGt, Np, Nu, 1, 3, std::move(e), std::move(f)));
+        NM_TRY(build_row_desc(P->EGt));
     }
 
     // ---- device inputs

@@ -70,53 +70,6 @@ __device__ __forceinline__ void kron_epilogue(const KronArgs<T>& a, int64_t row,
     }
 }
 
-template <typename T, int R, int CPT, int MODE>
-__global__ void __launch_bounds__(kThreads) kron_kernel(const KronArgs<T> a, int tpr_shift) {
-    const int tpr = 1 << tpr_shift;
-    const int lane = threadIdx.x & (tpr - 1);
-    const int64_t row = (int64_t)blockIdx.x * (kThreads >> tpr_shift) + (threadIdx.x >> tpr_shift);
-    if (row >= a.nrows) return;
-    T acc[CPT][R];
-#pragma unroll
-    for (int q = 0; q < CPT; ++q)
-#pragma unroll
-        for (int k = 0; k < R; ++k) acc[q][k] = T(0);
-    const int e0 = __ldg(a.rowptr + row), e1 = __ldg(a.rowptr + row + 1);
-    for (int e = e0; e < e1; ++e) {
-        const int64_t j = __ldg(a.col + e);
-        const T v = __ldg(a.val + e);
-        const T* xj = a.X + (int64_t)R * j * a.ldx;
-#pragma unroll
-        for (int q = 0; q < CPT; ++q) {
-            const int c = lane + q * tpr;
-            if (c < a.b) {
-#pragma unroll
-                for (int k = 0; k < R; ++k) acc[q][k] += v * __ldg(xj + k * a.ldx + c);
-            }
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < CPT; ++q) {
-        const int c = lane + q * tpr;
-        if (c >= a.b) continue;
-        kron_epilogue<T, R, MODE>(a, row, c, acc[q]);
-    }
-}
-
-template <typename T, int R, int MODE>
-static int kron_dispatch_cpt(int cpt, const KronArgs<T>& a, int shift, cudaStream_t s) {
-    const int rows_per_block = kThreads >> shift;
-    const int64_t grid = (a.nrows + rows_per_block - 1) / rows_per_block;
-    if (grid == 0) return NM_OK;
-    if (cpt == 1)
-        kron_kernel<T, R, 1, MODE><<<(unsigned)grid, kThreads, 0, s>>>(a, shift);
-    else
-        kron_kernel<T, R, 2, MODE><<<(unsigned)grid, kThreads, 0, s>>>(a, shift);
-    count_launch();
-    NM_CUDA(cudaGetLastError());
-    return NM_OK;
-}
-
 // Tiled variant for float blocks of exactly 32 columns (ld 32): one CTA per
 // tile of consecutive rows. The tile's distinct neighbour nodes (R x 32
 // floats each, 16-byte aligned runs) are copied into shared memory with
@@ -711,162 +664,22 @@ int launch_kron(int R, int mode, const KronArgs<T>& a, cudaStream_t s) {
             if (R == 1 && mode == KRON_CHEB) return kron_tile_launch<1, KRON_CHEB>(a, s);
         }
     }
-    if (a.b >= 17 && a.b <= 64) {
-        if (R == 3) {
-            switch (mode) {
-                case KRON_PLAIN: return kron_warp_launch<T, 3, KRON_PLAIN>(a, s);
-                case KRON_CHEB: return kron_warp_launch<T, 3, KRON_CHEB>(a, s);
-                case KRON_CHEB_FILT: return kron_warp_launch<T, 3, KRON_CHEB_FILT>(a, s);
-                case KRON_CORI: return kron_warp_launch<T, 3, KRON_CORI>(a, s);
-            }
-        } else if (R == 1 && mode == KRON_CHEB) {
-            return kron_warp_launch<T, 1, KRON_CHEB>(a, s);
-        }
-    }
-    const int shift = tpr_shift_for(a.b);
-    const int cpt = (a.b + (1 << shift) - 1) >> shift;
-    if (R == 3) {
-        switch (mode) {
-            case KRON_PLAIN: return kron_dispatch_cpt<T, 3, KRON_PLAIN>(cpt, a, shift, s);
-            case KRON_CHEB: return kron_dispatch_cpt<T, 3, KRON_CHEB>(cpt, a, shift, s);
-            case KRON_CHEB_FILT: return kron_dispatch_cpt<T, 3, KRON_CHEB_FILT>(cpt, a, shift, s);
-            case KRON_CORI: return kron_dispatch_cpt<T, 3, KRON_CORI>(cpt, a, shift, s);
-        }
-    } else if (R == 1) {
-        switch (mode) {
-            case KRON_PLAIN: return kron_dispatch_cpt<T, 1, KRON_PLAIN>(cpt, a, shift, s);
-            case KRON_CHEB: return kron_dispatch_cpt<T, 1, KRON_CHEB>(cpt, a, shift, s);
-            default: break;
-        }
-    }
-    return fail(NM_EINVAL, "unsupported kron mode");
-}
-
-// ----------------------------------------------------------------- 3x3 BSR
-template <typename T, int CPT>
-__global__ void __launch_bounds__(kThreads) bsr33_kernel(const Bsr33Args<T> a, int tpr_shift) {
-    const int tpr = 1 << tpr_shift;
-    const int lane = threadIdx.x & (tpr - 1);
-    const int64_t row = (int64_t)blockIdx.x * (kThreads >> tpr_shift) + (threadIdx.x >> tpr_shift);
-    if (row >= a.nrows) return;
-    T acc[CPT][3];
-#pragma unroll
-    for (int q = 0; q < CPT; ++q) acc[q][0] = acc[q][1] = acc[q][2] = T(0);
-    const int e0 = __ldg(a.rowptr + row), e1 = __ldg(a.rowptr + row + 1);
-    for (int e = e0; e < e1; ++e) {
-        const int64_t j = __ldg(a.col + e);
-        const T* K = a.val + 9 * (int64_t)e;
-        T k[9];
-#pragma unroll
-        for (int t = 0; t < 9; ++t) k[t] = __ldg(K + t);
-        const T* xj = a.X + 3 * j * a.ldx;
-#pragma unroll
-        for (int q = 0; q < CPT; ++q) {
-            const int c = lane + q * tpr;
-            if (c < a.b) {
-                const T x0 = __ldg(xj + c), x1 = __ldg(xj + a.ldx + c), x2 = __ldg(xj + 2 * a.ldx + c);
-                acc[q][0] += k[0] * x0 + k[1] * x1 + k[2] * x2;
-                acc[q][1] += k[3] * x0 + k[4] * x1 + k[5] * x2;
-                acc[q][2] += k[6] * x0 + k[7] * x1 + k[8] * x2;
-            }
-        }
-    }
-    if (a.e_rowptr) {
-        const int f0 = __ldg(a.e_rowptr + row), f1 = __ldg(a.e_rowptr + row + 1);
-        for (int e = f0; e < f1; ++e) {
-            const int64_t p = __ldg(a.e_col + e);
-            const T v0 = __ldg(a.e_val + 3 * (int64_t)e), v1 = __ldg(a.e_val + 3 * (int64_t)e + 1),
-                    v2 = __ldg(a.e_val + 3 * (int64_t)e + 2);
-#pragma unroll
-            for (int q = 0; q < CPT; ++q) {
-                const int c = lane + q * tpr;
-                if (c < a.b) {
-                    const T sv = __ldg(a.S + p * a.lds + c);
-                    acc[q][0] += v0 * sv;
-                    acc[q][1] += v1 * sv;
-                    acc[q][2] += v2 * sv;
+    if constexpr (std::is_same<T, float>::value) {
+        // option vec = 0: the chunked schedule's row code on a plain grid
+        if (!a.vec && a.b >= 17) {
+            if (R == 3) {
+                switch (mode) {
+                    case KRON_PLAIN: return kron_warp_launch<T, 3, KRON_PLAIN>(a, s);
+                    case KRON_CHEB: return kron_warp_launch<T, 3, KRON_CHEB>(a, s);
+                    case KRON_CHEB_FILT: return kron_warp_launch<T, 3, KRON_CHEB_FILT>(a, s);
+                    case KRON_CORI: return kron_warp_launch<T, 3, KRON_CORI>(a, s);
                 }
+            } else if (R == 1 && mode == KRON_CHEB) {
+                return kron_warp_launch<T, 1, KRON_CHEB>(a, s);
             }
         }
     }
-    const T d = a.X1 ? a.dinv[row] * a.inv_theta : T(0);
-#pragma unroll
-    for (int q = 0; q < CPT; ++q) {
-        const int c = lane + q * tpr;
-        if (c >= a.b) continue;
-#pragma unroll
-        for (int m = 0; m < 3; ++m) {
-            a.W[(3 * row + m) * a.ldw + c] = acc[q][m];
-            if (a.X1) a.X1[(3 * row + m) * a.ldx1 + c] = d * acc[q][m];
-        }
-    }
-}
-
-template <typename T>
-int launch_bsr33(const Bsr33Args<T>& a, cudaStream_t s) {
-    if (a.b < 1 || a.b > 64) return fail(NM_EINVAL, "block width must be in 1..64");
-    const int shift = tpr_shift_for(a.b);
-    const int cpt = (a.b + (1 << shift) - 1) >> shift;
-    const int rows_per_block = kThreads >> shift;
-    const int64_t grid = (a.nrows + rows_per_block - 1) / rows_per_block;
-    if (grid == 0) return NM_OK;
-    if (cpt == 1)
-        bsr33_kernel<T, 1><<<(unsigned)grid, kThreads, 0, s>>>(a, shift);
-    else
-        bsr33_kernel<T, 2><<<(unsigned)grid, kThreads, 0, s>>>(a, shift);
-    count_launch();
-    NM_CUDA(cudaGetLastError());
-    return NM_OK;
-}
-
-// ----------------------------------------------------------------- 1x3 BSR
-template <typename T, int CPT>
-__global__ void __launch_bounds__(kThreads) bsr13_kernel(const Bsr13Args<T> a, int tpr_shift) {
-    const int tpr = 1 << tpr_shift;
-    const int lane = threadIdx.x & (tpr - 1);
-    const int64_t row = (int64_t)blockIdx.x * (kThreads >> tpr_shift) + (threadIdx.x >> tpr_shift);
-    if (row >= a.nrows) return;
-    T acc[CPT];
-#pragma unroll
-    for (int q = 0; q < CPT; ++q) acc[q] = T(0);
-    const int e0 = __ldg(a.rowptr + row), e1 = __ldg(a.rowptr + row + 1);
-    for (int e = e0; e < e1; ++e) {
-        const int64_t j = __ldg(a.col + e);
-        const T v0 = __ldg(a.val + 3 * (int64_t)e), v1 = __ldg(a.val + 3 * (int64_t)e + 1),
-                v2 = __ldg(a.val + 3 * (int64_t)e + 2);
-        const T* xj = a.X + 3 * j * a.ldx;
-#pragma unroll
-        for (int q = 0; q < CPT; ++q) {
-            const int c = lane + q * tpr;
-            if (c < a.b)
-                acc[q] += v0 * __ldg(xj + c) + v1 * __ldg(xj + a.ldx + c) + v2 * __ldg(xj + 2 * a.ldx + c);
-        }
-    }
-    const T d = a.S1 ? a.dinv[row] * a.inv_theta : T(0);
-#pragma unroll
-    for (int q = 0; q < CPT; ++q) {
-        const int c = lane + q * tpr;
-        if (c >= a.b) continue;
-        a.Q[row * a.ldq + c] = acc[q];
-        if (a.S1) a.S1[row * a.lds1 + c] = d * acc[q];
-    }
-}
-
-template <typename T>
-int launch_bsr13(const Bsr13Args<T>& a, cudaStream_t s) {
-    if (a.b < 1 || a.b > 64) return fail(NM_EINVAL, "block width must be in 1..64");
-    const int shift = tpr_shift_for(a.b);
-    const int cpt = (a.b + (1 << shift) - 1) >> shift;
-    const int rows_per_block = kThreads >> shift;
-    const int64_t grid = (a.nrows + rows_per_block - 1) / rows_per_block;
-    if (grid == 0) return NM_OK;
-    if (cpt == 1)
-        bsr13_kernel<T, 1><<<(unsigned)grid, kThreads, 0, s>>>(a, shift);
-    else
-        bsr13_kernel<T, 2><<<(unsigned)grid, kThreads, 0, s>>>(a, shift);
-    count_launch();
-    NM_CUDA(cudaGetLastError());
-    return NM_OK;
+    return launch_kron_rows<T>(R, mode, a, s);
 }
 
 // ----------------------------------------------------------------- small kernels
@@ -1663,10 +1476,6 @@ int launch_philox_normal(int64_t count, uint64_t seed, double* out, cudaStream_t
 
 template int launch_kron<double>(int, int, const KronArgs<double>&, cudaStream_t);
 template int launch_kron<float>(int, int, const KronArgs<float>&, cudaStream_t);
-template int launch_bsr33<double>(const Bsr33Args<double>&, cudaStream_t);
-template int launch_bsr33<float>(const Bsr33Args<float>&, cudaStream_t);
-template int launch_bsr13<double>(const Bsr13Args<double>&, cudaStream_t);
-template int launch_bsr13<float>(const Bsr13Args<float>&, cudaStream_t);
 template int launch_dscale<double>(int, int64_t, int, double, const double*, const double*, int64_t, double*, int64_t, cudaStream_t);
 template int launch_dscale<float>(int, int64_t, int, float, const float*, const float*, int64_t, float*, int64_t, cudaStream_t);
 template int launch_scale_copy<double>(int64_t, int, double, const double*, int64_t, double*, int64_t, cudaStream_t);

@@ -54,6 +54,7 @@ struct Clusters {
 template <typename T>
 struct KronArgs {
     int nrows = 0;
+    const int4* desc = nullptr;   // rows in launch order: row, first entry, end
     const int* rowptr = nullptr;
     const int* col = nullptr;
     const T* val = nullptr;
@@ -121,6 +122,9 @@ int tma_status(int* err_dev, cudaStream_t s);
 
 template <typename T>
 int launch_kron(int R, int mode, const KronArgs<T>& a, cudaStream_t s);
+// The row-by-row form of it (rows.cu): any type, width and leading dimension.
+template <typename T>
+int launch_kron_rows(int R, int mode, const KronArgs<T>& a, cudaStream_t s);
 
 // W = A X (+ E S) for the 3x3-block CSR A over u-nodes and the optional
 // 3x1-block CSR E (u-nodes x p-nodes) applied to the pressure block S.
@@ -129,6 +133,7 @@ int launch_kron(int R, int mode, const KronArgs<T>& a, cudaStream_t s);
 template <typename T>
 struct Bsr33Args {
     int nrows = 0;
+    const int4* desc = nullptr;
     const int* rowptr = nullptr;
     const int* col = nullptr;
     const T* val = nullptr;
@@ -152,6 +157,7 @@ int launch_bsr33(const Bsr33Args<T>& a, cudaStream_t s);
 template <typename T>
 struct Bsr13Args {
     int nrows = 0;
+    const int4* desc = nullptr;
     const int* rowptr = nullptr;
     const int* col = nullptr;
     const T* val = nullptr;

@@ -75,6 +75,7 @@ struct DevCSR {
     DevBuf val;      // double [nnz * rb * cb]
     DevBuf val32;    // float  [nnz * rb * cb] (on demand): fl(val), the high part
     DevBuf vlo32;    // float  [nnz * rb * cb] (on demand): fl(val - fl(val)), the low part
+    DevBuf desc;     // int4 [nrows]: row, first entry, end, in launch order (rows.cu)
     DevBuf dinv;     // inverse diagonal (scalar square matrices only), double
     DevBuf dinv32;
     std::vector<int32_t> h_rowptr, h_col;   // host copy of the pattern
@@ -103,6 +104,7 @@ struct DevCSR {
 
 int build_tma_tiles(DevCSR& A, cudaStream_t s);
 int build_clusters(DevCSR& A, cudaStream_t s);
+int build_row_desc(DevCSR& A);
 
 struct Workspace {
     DevBuf buf;      // filter recurrence scratch

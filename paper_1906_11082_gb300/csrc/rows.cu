@@ -1,0 +1,628 @@
+// Sparse products row by row (any type, width and leading dimension): the
+// scalar matrix (x) I_R with the semi-iteration epilogues, the 3x3-block K_eff
+// product and the 1x3-block E_G^T product.
+//
+// What bounds them: in double, the FP64 units (2 multiply-adds per clock and
+// SM) once the rows fill the chip; on small meshes and narrow blocks the chain
+// of dependent loads row -> columns -> records, and the launch. So:
+//  - a row's entries are split over S lane groups and U entries per group are
+//    in flight together: a 27-entry row is fetched in one or two round trips;
+//    S falls to 1 as the rows fill the chip, since every doubling adds FP64
+//    additions;
+//  - an FP64 instruction holds its SM's pipe for 16 cycles however few lanes
+//    are active: the groups' sums are scattered, not broadcast, and the
+//    epilogue is spread over the groups with them;
+//  - rows are taken in order of length inside windows of 64 (descriptors row,
+//    first entry, end), so that the rows of one warp end together: unsorted,
+//    a warp of eight rows runs as long as its 65-entry vertex row while the
+//    mean is 27;
+//  - CTAs of two warps: with four, 1124 CTAs of equal speed left 60 for a
+//    second, nearly empty wave (the step's SMs were active 61% of the time);
+//  - kernels of a chain start while their predecessor drains (programmatic
+//    dependent launch): descriptors, columns and values do not depend on it
+//    and are loaded before the wait.
+// A lane group per row walking its entries one by one (the form before)
+// against now, per semi-iteration step in double at 8 columns: 633 rows
+// 26 -> 6.4 us, 17,977 rows 49 -> 40 us (FP64 floor 20 us).
+#include <algorithm>
+#include <atomic>
+#include <cstdint>
+#include <initializer_list>
+#include <vector>
+
+#include "kernels.h"
+#include "nm_internal.h"
+
+namespace nm {
+
+namespace {
+
+constexpr int kThreads = 64;
+constexpr int kWindow = 64;
+
+// VW consecutive values (16-byte aligned when VW = 2 doubles / 8 when 2 floats)
+template <typename T, int VW>
+struct Vec {
+    T v[VW];
+};
+template <typename T, int VW>
+__device__ __forceinline__ Vec<T, VW> ld(const T* p) {
+    Vec<T, VW> r;
+    if constexpr (VW == 1) {
+        r.v[0] = *p;
+    } else if constexpr (sizeof(T) == 8) {
+        const double2 t = *reinterpret_cast<const double2*>(p);
+        r.v[0] = t.x, r.v[1] = t.y;
+    } else {
+        const float2 t = *reinterpret_cast<const float2*>(p);
+        r.v[0] = t.x, r.v[1] = t.y;
+    }
+    return r;
+}
+template <typename T, int VW>
+__device__ __forceinline__ void st(T* p, const Vec<T, VW>& r) {
+    if constexpr (VW == 1) {
+        *p = r.v[0];
+    } else if constexpr (sizeof(T) == 8) {
+        *reinterpret_cast<double2*>(p) = make_double2(r.v[0], r.v[1]);
+    } else {
+        *reinterpret_cast<float2*>(p) = make_float2(r.v[0], r.v[1]);
+    }
+}
+template <typename T, int VW>
+__device__ __forceinline__ Vec<T, VW> zero() {
+    Vec<T, VW> r;
+#pragma unroll
+    for (int i = 0; i < VW; ++i) r.v[i] = T(0);
+    return r;
+}
+
+// Wait for the predecessor's results, then let the successor start: only two
+// kernels of a chain are ever in flight together. What is loaded before this
+// point is matrix data no kernel of a chain writes; blocks are read after it,
+// by plain (not read-only path) loads.
+__device__ __forceinline__ void dep_sync() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Sums N values over the S lane groups (tl lanes each) of a row. Every step
+// halves the values a lane keeps (a group gives away the half it drops), so
+// that S groups cost about N additions, not N log2 S, and what follows the
+// sum is spread over the groups: on return v[0 .. cnt) holds the sums of the
+// values base .. base + cnt - 1. An FP64 instruction holds its SM's pipe for
+// 16 cycles however few lanes are active.
+template <typename T, int N, int S>
+struct Scatter {
+    // values a lane keeps at most
+    static constexpr int kept(int n, int s) { return s == 1 || n == 1 ? n : kept((n + 1) / 2, s / 2); }
+    static constexpr int kKeep = kept(N, S);
+    int base = 0, cnt = N;
+    __device__ __forceinline__ explicit Scatter(int sp) {
+        int n = N;
+#pragma unroll
+        for (int m = 1; m < S; m *= 2) {
+            const bool up = sp & m;
+            if (n == 1) {
+                if (up) cnt = 0;
+            } else {
+                const int h = (n + 1) / 2;
+                base += up ? h : 0;
+                cnt = up ? max(cnt - h, 0) : min(cnt, h);
+                n = h;
+            }
+        }
+    }
+    __device__ __forceinline__ void sum(T (&v)[N], int sp, int tl) const {
+        int n = N;
+#pragma unroll
+        for (int m = 1; m < S; m *= 2) {
+            const bool up = sp & m;
+            if (n == 1) {
+                v[0] += __shfl_xor_sync(0xffffffffu, v[0], m * tl);
+            } else {
+                const int h = (n + 1) / 2;
+#pragma unroll
+                for (int i = 0; i < (N + 1) / 2; ++i) {
+                    if (i < h) {
+                        const T hi = h + i < n ? v[h + i < N ? h + i : 0] : T(0);
+                        const T give = up ? v[i] : hi, keep = up ? hi : v[i];
+                        v[i] = keep + __shfl_xor_sync(0xffffffffu, give, m * tl);
+                    }
+                }
+                n = h;
+            }
+        }
+    }
+};
+
+// Where a lane works: lane q of split sp of row slot `slot`; column c (of
+// VW), valid columns only where on.
+struct Place {
+    int sp, c;
+    bool on;
+    int4 d;   // row, first entry, end
+};
+template <int VW, int S>
+__device__ __forceinline__ Place place(const int4* desc, int nrows, int b, int tl_shift) {
+    Place p;
+    const int t = blockIdx.x * kThreads + threadIdx.x;
+    const int slot = t >> tl_shift >> (S == 1 ? 0 : S == 2 ? 1 : S == 4 ? 2 : 3);
+    p.sp = (t >> tl_shift) & (S - 1);
+    p.c = VW * ((t & ((1 << tl_shift) - 1)) + (blockIdx.y << tl_shift));
+    p.on = slot < nrows && p.c < b;
+    p.d = __ldg(desc + min(slot, nrows - 1));
+    if (!p.on) p.d.z = p.d.y;   // no entries
+    return p;
+}
+
+}  // namespace
+
+// ----------------------------------------------------------------- A (x) I_R
+template <typename T, int R, int MODE, int VW, int S, int U>
+__global__ void __launch_bounds__(kThreads) kron_rows_kernel(const KronArgs<T> a, int tl_shift) {
+    const Place p = place<VW, S>(a.desc, a.nrows, a.b, tl_shift);
+    const int c = p.on ? p.c : 0;
+    const int64_t row = p.d.x;
+    T acc[R * VW];
+#pragma unroll
+    for (int i = 0; i < R * VW; ++i) acc[i] = T(0);
+    const T* const X = a.X + c;
+    const int64_t RL = (int64_t)R * a.ldx;
+    int e = p.d.y + p.sp;
+    int j[U];
+    T v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const bool ok = e + u * S < p.d.z;
+        j[u] = ok ? __ldg(a.col + e + u * S) : -1;
+        v[u] = ok ? __ldg(a.val + e + u * S) : T(0);
+    }
+    constexpr bool kCheb = MODE == KRON_CHEB || MODE == KRON_CHEB_FILT;
+    const T dd = kCheb ? __ldg(a.dinv + row) * a.inv_theta : T(0);
+    dep_sync();
+    constexpr int N = R * VW;
+    // CORI mixes the components: its lanes keep all of them
+    constexpr int SS = MODE == KRON_CORI ? 1 : S;
+    const Scatter<T, N, SS> sc(p.sp);
+    constexpr int K = Scatter<T, N, SS>::kKeep;
+    const int cnt = p.on ? sc.cnt : 0;
+    // a lane's own values of a block: whole vectors, or single ones when the
+    // row's sums are scattered over its lane groups
+    auto own = [&](const T* base, int64_t l, T (&o)[K]) {
+        if constexpr (SS == 1) {
+#pragma unroll
+            for (int k = 0; k < R; ++k) {
+                const Vec<T, VW> t = p.on ? ld<T, VW>(base + (R * row + k) * l + c) : zero<T, VW>();
+#pragma unroll
+                for (int i = 0; i < VW; ++i) o[k * VW + i] = t.v[i];
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < K; ++i) {
+                const int t = sc.base + i;
+                o[i] = i < cnt ? base[(R * row + t / VW) * l + c + t % VW] : T(0);
+            }
+        }
+    };
+    auto put = [&](T* base, int64_t l, const T (&o)[K]) {
+        if constexpr (SS == 1) {
+            if (p.on && (S == 1 || p.sp == 0))
+#pragma unroll
+                for (int k = 0; k < R; ++k) {
+                    Vec<T, VW> t;
+#pragma unroll
+                    for (int i = 0; i < VW; ++i) t.v[i] = o[k * VW + i];
+                    st<T, VW>(base + (R * row + k) * l + c, t);
+                }
+        } else {
+#pragma unroll
+            for (int i = 0; i < K; ++i) {
+                const int t = sc.base + i;
+                if (i < cnt) base[(R * row + t / VW) * l + c + t % VW] = o[i];
+            }
+        }
+    };
+    T xk[K], w[K], xp[K];
+    if (kCheb) {
+        own(a.X, a.ldx, xk);
+        own(a.W, a.ldw, w);
+#pragma unroll
+        for (int i = 0; i < K; ++i) xp[i] = T(0);
+        if (a.Xp) own(a.Xp, a.ldp, xp);
+    }
+    while (e < p.d.z) {
+        Vec<T, VW> x[U][R];
+        T vc[U];
+        bool in[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            in[u] = j[u] >= 0;
+            vc[u] = v[u];
+#pragma unroll
+            for (int k = 0; k < R; ++k) x[u][k] = in[u] ? ld<T, VW>(X + j[u] * RL + k * a.ldx) : zero<T, VW>();
+        }
+        e += U * S;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const bool ok = e + u * S < p.d.z;
+            j[u] = ok ? __ldg(a.col + e + u * S) : -1;
+            v[u] = ok ? __ldg(a.val + e + u * S) : T(0);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (in[u]) {
+#pragma unroll
+                for (int k = 0; k < R; ++k)
+#pragma unroll
+                    for (int i = 0; i < VW; ++i) acc[k * VW + i] = fma(vc[u], x[u][k].v[i], acc[k * VW + i]);
+            }
+    }
+    if constexpr (SS == S) {
+        sc.sum(acc, p.sp, 1 << tl_shift);
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+#pragma unroll
+            for (int m = 1; m < S; m *= 2) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], m << tl_shift);
+    }
+    T o[K];
+    if (MODE == KRON_PLAIN) {
+#pragma unroll
+        for (int i = 0; i < K; ++i) o[i] = acc[i];
+        put(a.Y, a.ldy, o);
+    } else if constexpr (MODE == KRON_CORI) {
+#pragma unroll
+        for (int m = 0; m < R; ++m)
+#pragma unroll
+            for (int i = 0; i < VW; ++i) {
+                T y = T(0);
+#pragma unroll
+                for (int k = 0; k < R; ++k) y += a.sk[m * 3 + k] * acc[k * VW + i];
+                o[m * VW + i] = y;
+            }
+        put(a.Y, a.ldy, o);
+    } else {
+#pragma unroll
+        for (int i = 0; i < K; ++i) o[i] = xp[i] + a.om * (xk[i] - xp[i] + dd * (w[i] - acc[i]));
+        if (MODE == KRON_CHEB) {
+            put(a.Xn, a.ldn, o);
+        } else {
+            T tk[K], tp[K];
+            own(a.Tk, a.ldtk, tk);
+#pragma unroll
+            for (int i = 0; i < K; ++i) tp[i] = T(0);
+            if (a.Tp) own(a.Tp, a.ldtp, tp);
+#pragma unroll
+            for (int i = 0; i < K; ++i) o[i] = a.a1 * (o[i] - a.cshift * tk[i]) - a.a2 * tp[i];
+            put(a.Tn, a.ldtn, o);
+            if (a.Z) {
+                T z[K];
+                own(a.Z, a.ldz, z);
+#pragma unroll
+                for (int i = 0; i < K; ++i) {
+                    const int cc = c + (SS == 1 ? i : sc.base + i) % VW;
+                    z[i] += (a.gam_tab && cc < a.b ? (T)a.gam_tab[cc / a.gam_group] : a.gam) * o[i];
+                }
+                put(a.Z, a.ldz, z);
+            }
+        }
+    }
+}
+
+// ----------------------------------------------------------------- 3x3 BSR (+ E S)
+template <typename T, int VW, int S, int U>
+__global__ void __launch_bounds__(kThreads) bsr33_rows_kernel(const Bsr33Args<T> a, int tl_shift) {
+    const Place p = place<VW, S>(a.desc, a.nrows, a.b, tl_shift);
+    const int c = p.on ? p.c : 0;
+    const int64_t row = p.d.x;
+    const int f0 = a.e_rowptr && p.on ? __ldg(a.e_rowptr + row) : 0, f1 = a.e_rowptr && p.on ? __ldg(a.e_rowptr + row + 1) : 0;
+    constexpr int N = 3 * VW;
+    T acc[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) acc[i] = T(0);
+    const T* const X = a.X + c;
+    int e = p.d.y + p.sp;
+    int j[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) j[u] = e + u * S < p.d.z ? __ldg(a.col + e + u * S) : -1;
+    dep_sync();
+    while (e < p.d.z) {
+        Vec<T, VW> x[U][3];
+        T kv[U][9];
+        bool in[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            in[u] = j[u] >= 0;
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                x[u][k] = in[u] ? ld<T, VW>(X + (3 * (int64_t)j[u] + k) * a.ldx) : zero<T, VW>();
+#pragma unroll
+            for (int t = 0; t < 9; ++t) kv[u][t] = in[u] ? __ldg(a.val + 9 * (int64_t)(e + u * S) + t) : T(0);
+        }
+        e += U * S;
+#pragma unroll
+        for (int u = 0; u < U; ++u) j[u] = e + u * S < p.d.z ? __ldg(a.col + e + u * S) : -1;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (in[u]) {
+#pragma unroll
+                for (int m = 0; m < 3; ++m)
+#pragma unroll
+                    for (int k = 0; k < 3; ++k)
+#pragma unroll
+                        for (int i = 0; i < VW; ++i)
+                            acc[m * VW + i] = fma(kv[u][3 * m + k], x[u][k].v[i], acc[m * VW + i]);
+            }
+    }
+#pragma unroll 2
+    for (int f = f0 + p.sp; f < f1; f += S) {
+        const Vec<T, VW> sv = ld<T, VW>(a.S + (int64_t)__ldg(a.e_col + f) * a.lds + c);
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            const T ev = __ldg(a.e_val + 3 * (int64_t)f + m);
+#pragma unroll
+            for (int i = 0; i < VW; ++i) acc[m * VW + i] = fma(ev, sv.v[i], acc[m * VW + i]);
+        }
+    }
+    const Scatter<T, N, S> sc(p.sp);
+    constexpr int K = Scatter<T, N, S>::kKeep;
+    sc.sum(acc, p.sp, 1 << tl_shift);
+    if (!p.on) return;
+    const T d = a.X1 ? __ldg(a.dinv + row) * a.inv_theta : T(0);
+    if constexpr (S == 1) {
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            Vec<T, VW> t;
+#pragma unroll
+            for (int i = 0; i < VW; ++i) t.v[i] = acc[m * VW + i];
+            st<T, VW>(a.W + (3 * row + m) * a.ldw + c, t);
+            if (a.X1) {
+#pragma unroll
+                for (int i = 0; i < VW; ++i) t.v[i] *= d;
+                st<T, VW>(a.X1 + (3 * row + m) * a.ldx1 + c, t);
+            }
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < K; ++i) {
+            if (i >= sc.cnt) break;
+            const int t = sc.base + i;
+            a.W[(3 * row + t / VW) * a.ldw + c + t % VW] = acc[i];
+            if (a.X1) a.X1[(3 * row + t / VW) * a.ldx1 + c + t % VW] = d * acc[i];
+        }
+    }
+}
+
+// ----------------------------------------------------------------- 1x3 BSR
+template <typename T, int VW, int S, int U>
+__global__ void __launch_bounds__(kThreads) bsr13_rows_kernel(const Bsr13Args<T> a, int tl_shift) {
+    const Place p = place<VW, S>(a.desc, a.nrows, a.b, tl_shift);
+    const int c = p.on ? p.c : 0;
+    const int64_t row = p.d.x;
+    T acc[VW];
+#pragma unroll
+    for (int i = 0; i < VW; ++i) acc[i] = T(0);
+    const T* const X = a.X + c;
+    int e = p.d.y + p.sp;
+    int j[U];
+    T v[U][3];
+    auto fetch = [&]() {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const bool ok = e + u * S < p.d.z;
+            j[u] = ok ? __ldg(a.col + e + u * S) : -1;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) v[u][k] = ok ? __ldg(a.val + 3 * (int64_t)(e + u * S) + k) : T(0);
+        }
+    };
+    fetch();
+    dep_sync();
+    while (e < p.d.z) {
+        Vec<T, VW> x[U][3];
+        T vc[U][3];
+        bool in[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) in[u] = j[u] >= 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                x[u][k] = in[u] ? ld<T, VW>(X + (3 * (int64_t)j[u] + k) * a.ldx) : zero<T, VW>();
+                vc[u][k] = v[u][k];
+            }
+        e += U * S;
+        fetch();
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (in[u]) {
+#pragma unroll
+                for (int k = 0; k < 3; ++k)
+#pragma unroll
+                    for (int i = 0; i < VW; ++i) acc[i] = fma(vc[u][k], x[u][k].v[i], acc[i]);
+            }
+    }
+    const Scatter<T, VW, S> sc(p.sp);
+    constexpr int K = Scatter<T, VW, S>::kKeep;
+    sc.sum(acc, p.sp, 1 << tl_shift);
+    if (!p.on) return;
+    const T d = a.S1 ? __ldg(a.dinv + row) * a.inv_theta : T(0);
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+        if (i >= sc.cnt) break;
+        a.Q[row * a.ldq + c + sc.base + i] = acc[i];
+        if (a.S1) a.S1[row * a.lds1 + c + sc.base + i] = d * acc[i];
+    }
+}
+
+// ----------------------------------------------------------------- launches
+namespace {
+
+struct Shape {
+    int tl_shift, splits;
+    dim3 grid;
+};
+
+// tl lanes (a power of two, at most 32) cover the columns, chunks of 32 VW
+// columns go to the grid's y; the splits double while the rows leave the chip
+// below 16 warps per SM (a double filter at 17,977 rows and 8 columns: 16.6 /
+// 15.1 / 11.7 / 12.1 ms with 4 / 8 / 16 / 32 warps).
+Shape shape(int nrows, int b, int vw) {
+    static std::atomic<int> sm_count{0};
+    int sms = sm_count.load(std::memory_order_relaxed);
+    if (sms == 0) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+            sms = 148;
+        sm_count.store(sms, std::memory_order_relaxed);
+    }
+    const int lanes = (b + vw - 1) / vw;
+    Shape h;
+    h.tl_shift = 0;
+    while (h.tl_shift < 5 && (1 << h.tl_shift) < lanes) ++h.tl_shift;
+    const int ny = (lanes + (1 << h.tl_shift) - 1) >> h.tl_shift;
+    h.splits = 1;
+    while (h.splits < 8 && (h.splits << h.tl_shift) < 32 &&
+           ((((int64_t)nrows * ny * h.splits) << h.tl_shift) >> 5) < 16 * (int64_t)sms)
+        h.splits *= 2;
+    const int64_t threads = ((int64_t)nrows * h.splits) << h.tl_shift;
+    h.grid = dim3((unsigned)((threads + kThreads - 1) / kThreads), (unsigned)ny);
+    return h;
+}
+
+template <typename... A>
+int launch(void (*k)(A...), const Shape& h, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = h.grid;
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    NM_CUDA(cudaLaunchKernelEx(&cfg, k, args...));
+    count_launch();
+    return NM_OK;
+}
+
+template <typename T, int R, int MODE, int VW>
+int kron_rows_go(const KronArgs<T>& a, cudaStream_t s) {
+    const Shape h = shape(a.nrows, a.b, VW);
+    constexpr int U = 4;
+    switch (h.splits) {
+        case 1: return launch(kron_rows_kernel<T, R, MODE, VW, 1, U>, h, s, a, h.tl_shift);
+        case 2: return launch(kron_rows_kernel<T, R, MODE, VW, 2, U>, h, s, a, h.tl_shift);
+        case 4: return launch(kron_rows_kernel<T, R, MODE, VW, 4, U>, h, s, a, h.tl_shift);
+        default: return launch(kron_rows_kernel<T, R, MODE, VW, 8, U>, h, s, a, h.tl_shift);
+    }
+}
+
+// two columns per lane need even widths and strides and aligned operands
+template <typename T>
+bool pairs(int b, std::initializer_list<int64_t> lds, std::initializer_list<const void*> ptrs) {
+    if (b % 2) return false;
+    for (int64_t l : lds)
+        if (l % 2) return false;
+    uintptr_t p = 0;
+    for (const void* q : ptrs) p |= (uintptr_t)q;
+    return (p & (2 * sizeof(T) - 1)) == 0;
+}
+
+template <typename T, int R, int MODE>
+int kron_rows_mode(const KronArgs<T>& a, cudaStream_t s) {
+    if (a.nrows == 0) return NM_OK;
+    bool two;
+    if (MODE == KRON_PLAIN || MODE == KRON_CORI)
+        two = pairs<T>(a.b, {a.ldx, a.ldy}, {a.X, a.Y});
+    else if (MODE == KRON_CHEB)
+        two = pairs<T>(a.b, {a.ldx, a.ldw, a.ldp, a.ldn}, {a.X, a.W, a.Xp, a.Xn});
+    else
+        two = pairs<T>(a.b, {a.ldx, a.ldw, a.ldp, a.ldtk, a.ldtp, a.ldtn, a.ldz}, {a.X, a.W, a.Xp, a.Tk, a.Tp, a.Tn, a.Z});
+    return two ? kron_rows_go<T, R, MODE, 2>(a, s) : kron_rows_go<T, R, MODE, 1>(a, s);
+}
+
+template <typename T, int VW>
+int bsr33_rows_go(const Bsr33Args<T>& a, cudaStream_t s) {
+    const Shape h = shape(a.nrows, a.b, VW);
+    switch (h.splits) {
+        case 1: return launch(bsr33_rows_kernel<T, VW, 1, 2>, h, s, a, h.tl_shift);
+        case 2: return launch(bsr33_rows_kernel<T, VW, 2, 2>, h, s, a, h.tl_shift);
+        case 4: return launch(bsr33_rows_kernel<T, VW, 4, 2>, h, s, a, h.tl_shift);
+        default: return launch(bsr33_rows_kernel<T, VW, 8, 2>, h, s, a, h.tl_shift);
+    }
+}
+
+template <typename T, int VW>
+int bsr13_rows_go(const Bsr13Args<T>& a, cudaStream_t s) {
+    const Shape h = shape(a.nrows, a.b, VW);
+    switch (h.splits) {
+        case 1: return launch(bsr13_rows_kernel<T, VW, 1, 4>, h, s, a, h.tl_shift);
+        case 2: return launch(bsr13_rows_kernel<T, VW, 2, 4>, h, s, a, h.tl_shift);
+        case 4: return launch(bsr13_rows_kernel<T, VW, 4, 4>, h, s, a, h.tl_shift);
+        default: return launch(bsr13_rows_kernel<T, VW, 8, 4>, h, s, a, h.tl_shift);
+    }
+}
+
+}  // namespace
+
+template <typename T>
+int launch_kron_rows(int R, int mode, const KronArgs<T>& a, cudaStream_t s) {
+    if (R == 3) {
+        switch (mode) {
+            case KRON_PLAIN: return kron_rows_mode<T, 3, KRON_PLAIN>(a, s);
+            case KRON_CHEB: return kron_rows_mode<T, 3, KRON_CHEB>(a, s);
+            case KRON_CHEB_FILT: return kron_rows_mode<T, 3, KRON_CHEB_FILT>(a, s);
+            case KRON_CORI: return kron_rows_mode<T, 3, KRON_CORI>(a, s);
+        }
+    } else if (R == 1) {
+        switch (mode) {
+            case KRON_PLAIN: return kron_rows_mode<T, 1, KRON_PLAIN>(a, s);
+            case KRON_CHEB: return kron_rows_mode<T, 1, KRON_CHEB>(a, s);
+            default: break;
+        }
+    }
+    return fail(NM_EINVAL, "unsupported kron mode");
+}
+
+template <typename T>
+int launch_bsr33(const Bsr33Args<T>& a, cudaStream_t s) {
+    if (a.b < 1 || a.b > 64) return fail(NM_EINVAL, "block width must be in 1..64");
+    if (a.nrows == 0) return NM_OK;
+    return pairs<T>(a.b, {a.ldx, a.ldw, a.lds, a.ldx1}, {a.X, a.W, a.S, a.X1}) ? bsr33_rows_go<T, 2>(a, s)
+                                                                             : bsr33_rows_go<T, 1>(a, s);
+}
+
+template <typename T>
+int launch_bsr13(const Bsr13Args<T>& a, cudaStream_t s) {
+    if (a.b < 1 || a.b > 64) return fail(NM_EINVAL, "block width must be in 1..64");
+    if (a.nrows == 0) return NM_OK;
+    return pairs<T>(a.b, {a.ldx, a.ldq, a.lds1}, {a.X, a.Q, a.S1}) ? bsr13_rows_go<T, 2>(a, s)
+                                                                  : bsr13_rows_go<T, 1>(a, s);
+}
+
+// Row descriptors: rows of each window of 64 in order of decreasing length.
+int build_row_desc(DevCSR& A) {
+    const int64_t N = A.nrows;
+    std::vector<int4> d(std::max<int64_t>(N, 1));
+    const int32_t* rp = A.h_rowptr.data();
+#pragma omp parallel for schedule(static)
+    for (int64_t w = 0; w < (N + kWindow - 1) / kWindow; ++w) {
+        const int64_t r0 = w * kWindow, r1 = std::min<int64_t>(N, r0 + kWindow);
+        for (int64_t r = r0; r < r1; ++r) d[r] = make_int4((int)r, rp[r], rp[r + 1], 0);
+        std::stable_sort(d.begin() + r0, d.begin() + r1, [](const int4& x, const int4& y) { return x.z - x.y > y.z - y.y; });
+    }
+    NM_TRY(A.desc.alloc(d.size() * sizeof(int4)));
+    NM_CUDA(cudaMemcpy(A.desc.p, d.data(), d.size() * sizeof(int4), cudaMemcpyHostToDevice));
+    return NM_OK;
+}
+
+template int launch_kron_rows<double>(int, int, const KronArgs<double>&, cudaStream_t);
+template int launch_kron_rows<float>(int, int, const KronArgs<float>&, cudaStream_t);
+template int launch_bsr33<double>(const Bsr33Args<double>&, cudaStream_t);
+template int launch_bsr33<float>(const Bsr33Args<float>&, cudaStream_t);
+template int launch_bsr13<double>(const Bsr13Args<double>&, cudaStream_t);
+template int launch_bsr13<float>(const Bsr13Args<float>&, cudaStream_t);
+
+}  // namespace nm

@@ -40,6 +40,7 @@ struct Mats {
     const T* EG = nullptr;
     const int *et_rp = nullptr, *et_col = nullptr;
     const T* EGt = nullptr;
+    const int4 *u_desc = nullptr, *p_desc = nullptr, *et_desc = nullptr;
     const DevCSR* Mcsr = nullptr;
     const DevCSR* Pcsr = nullptr;
     nm_problem* P = nullptr;
@@ -68,6 +69,7 @@ static Mats<T> mats(nm_problem* P) {
     m.AG = vals<T>(P->AG);
     m.Mr = vals<T>(P->Mr);
     m.dM = dinv<T>(P->Mr);
+    m.u_desc = P->Mr.desc.as<int4>();
     m.Mcsr = &P->Mr;
     m.Pcsr = &P->Pn;
     m.P = P;
@@ -82,6 +84,8 @@ static Mats<T> mats(nm_problem* P) {
         m.et_rp = P->EGt.rowptr.as<int>();
         m.et_col = P->EGt.col.as<int>();
         m.EGt = vals<T>(P->EGt);
+        m.p_desc = P->Pn.desc.as<int4>();
+        m.et_desc = P->EGt.desc.as<int4>();
     }
     return m;
 }
@@ -164,6 +168,7 @@ static int schur_pressure(const Mats<T>& m, const T* X, int64_t ldx, int b, int 
     ChebCoef cc(lo, hi);
     Bsr13Args<T> q;
     q.nrows = (int)m.Np;
+    q.desc = m.et_desc;
     q.rowptr = m.et_rp;
     q.col = m.et_col;
     q.val = m.EGt;
@@ -183,6 +188,7 @@ static int schur_pressure(const Mats<T>& m, const T* X, int64_t ldx, int b, int 
         om = 1.0 / (1.0 - om / cc.four_sig2);
         KronArgs<T> a;
         a.nrows = (int)m.Np;
+        a.desc = m.p_desc;
         a.rowptr = m.p_rp;
         a.col = m.p_col;
         a.val = m.Pn;
@@ -214,6 +220,7 @@ static int apply_K_t(nm_problem* P, const T* X, int64_t ldx, T* W, int64_t ldw, 
     Mats<T> m = mats<T>(P);
     Bsr33Args<T> a;
     a.nrows = (int)m.Nu;
+    a.desc = m.u_desc;
     a.rowptr = m.u_rp;
     a.col = m.u_col;
     a.val = m.AG;
@@ -277,6 +284,7 @@ static int mass_steps(const Mats<T>& m, int b, int k_M, double lo, double hi, co
         om = 1.0 / (1.0 - om / cc.four_sig2);
         KronArgs<T> a;
         a.nrows = (int)m.Nu;
+        a.desc = m.u_desc;
         a.rowptr = m.u_rp;
         a.col = m.u_col;
         a.val = m.Mr;
@@ -441,6 +449,7 @@ static int cheb32(nm_problem* P, const DevCSR& A, int R, int b, int k, double lo
         om = 1.0 / (1.0 - om / cc.four_sig2);
         KronArgs<float> a;
         a.nrows = (int)nodes;
+        a.desc = A.desc.as<int4>();
         a.rowptr = A.rowptr.as<int>();
         a.col = A.col.as<int>();
         a.val = A.val32.as<float>();
@@ -531,6 +540,7 @@ static int apply_K_mixed_core(nm_problem* P, const double* X, int64_t ldx, doubl
     if (df && !pre_split) NM_TRY(launch_split(P->info.n, b, S.bp, X, ldx, S.Th, S.Tl, s));
     Bsr33Args<double> a;
     a.nrows = (int)m.Nu;
+    a.desc = m.u_desc;
     a.rowptr = m.u_rp;
     a.col = m.u_col;
     a.val = m.AG;
@@ -559,6 +569,7 @@ static int apply_K_mixed_core(nm_problem* P, const double* X, int64_t ldx, doubl
     if (m.Np > 0) {
         Bsr13Args<double> q;
         q.nrows = (int)m.Np;
+        q.desc = m.et_desc;
         q.rowptr = m.et_rp;
         q.col = m.et_col;
         q.val = m.EGt;
@@ -873,6 +884,7 @@ int apply_M_pub(nm_problem* P, const T* X, int64_t ldx, T* Y, int64_t ldy, int b
     Mats<T> m = mats<T>(P);
     KronArgs<T> a;
     a.nrows = (int)m.Nu;
+    a.desc = m.u_desc;
     a.rowptr = m.u_rp;
     a.col = m.u_col;
     a.val = m.Mr;

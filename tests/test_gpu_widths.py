@@ -57,6 +57,30 @@ def test_mixed_solve_every_width(nm, planet, b):
     assert rel_err(to_canonical(P, _host(X)), filtlan.refined_solve(S.M, 1.0 / S.M.diagonal(), Wc, 28)) <= 1e-11
 
 
+@pytest.mark.parametrize("b,ld", [(1, 1), (2, 2), (3, 4), (8, 8), (16, 17), (31, 31), (34, 34), (63, 63), (64, 66)])
+def test_double_rows_every_width(planet, b, ld):
+    """Row-by-row kernels: one and two columns per lane, one and two column
+    chunks, every split of a row's entries; the outer update and the pressure
+    chain inside a filter of degree 2; M, R and K products."""
+    S, P = planet
+    X = torch.zeros((S.n, ld), dtype=torch.float64, device=DEV)
+    Xc = np.random.default_rng(b).standard_normal((S.n, b))
+    X[:, :b] = _dev(to_internal(P, Xc))
+    op = filtlan.Operator(S, k_M=8, k_P=8)
+    lo, hi = filtlan.spectrum_bounds(op, S.n)
+    gam, c, e = filtlan.filter_coeffs(lo, hi, 0.5, 9.0, 2)
+    Y = torch.full_like(X, 7.0)
+    P.filter_apply(gam, c, e, 8, X[:, :b], Y[:, :b], k_P=8)
+    assert rel_err(to_canonical(P, _host(Y[:, :b])), filtlan.filter_apply(op, gam, c, e, Xc)) <= 1e-11
+    P.apply_K(X[:, :b], Y[:, :b], k_P=8)
+    assert rel_err(to_canonical(P, _host(Y[:, :b])), op.K(Xc)) <= 1e-11
+    P.apply_M(X[:, :b], Y[:, :b])
+    assert rel_err(to_canonical(P, _host(Y[:, :b])), S.M @ Xc) <= 1e-12
+    P.apply_R(X[:, :b], Y[:, :b])
+    assert rel_err(to_canonical(P, _host(Y[:, :b])), S.R @ Xc) <= 1e-12
+    assert bool((Y[:, b:] == 7.0).all())
+
+
 @pytest.mark.parametrize("b", [4, 21, 40, 64])
 def test_float_filter_widths(nm, planet, b):
     """The last float step carries the outer Chebyshev update; two column
