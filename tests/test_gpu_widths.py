@@ -124,3 +124,26 @@ def test_mixed_solve_on_the_ball(nm, ctx):
     X = torch.empty((S.n, 24), dtype=torch.float64, device=DEV)
     P.solve_M(_dev(to_internal(P, Wc)), X, k_M=28, prec=nm.NM_MIXED)
     assert rel_err(to_canonical(P, _host(X)), filtlan.refined_solve(S.M, 1.0 / S.M.diagonal(), Wc, 28)) <= 1e-11
+
+
+@pytest.mark.parametrize("I,J,K,pad", [(1, 1, 1, 0), (130, 9, 130, 1), (127, 33, 64, 1), (129, 16, 65, 2), (16, 8, 1000, 3)])
+def test_split_products_odd_strides(nm, ctx, I, J, K, pad):
+    """Dense products at the edges of their tiles (128 rows, 8 / 16 / 32
+    columns, 64 terms), with strides and bases that rule out 16-byte copies,
+    rows spread over 40 binades. Each kept or dropped piece errs by at most
+    2^-50 of the product of the largest entries of its row and column."""
+    rng = np.random.default_rng(I + J)
+    X, Y = rng.standard_normal((K, I + pad)), rng.standard_normal((K, J + pad))
+    X *= 2.0 ** rng.integers(-20, 20, (1, I + pad))
+    C = torch.zeros((J, I + pad), dtype=torch.float64, device=DEV)
+    dX, dY = _dev(X)[:, pad:], _dev(Y)[:, pad:]
+    ctx.gemm_tn(dX, dY, C)
+    bound = K * 2.0 ** -50 * np.outer(np.abs(X[:, pad:]).max(0), np.abs(Y[:, pad:]).max(0))
+    assert (np.abs(_host(C)[:, :I].T - X[:, pad:].T @ Y[:, pad:]) <= bound).all()
+    A, B = rng.standard_normal((I, K + pad)), rng.standard_normal((J, K + pad))
+    A *= 2.0 ** rng.integers(-20, 20, (I, 1))
+    D = torch.full((I, J + pad), 3.0, dtype=torch.float64, device=DEV)
+    ctx.gemm_nn(_dev(A)[:, pad:], _dev(B)[:, pad:], D[:, :J], beta=1.0)
+    bound = K * 2.0 ** -50 * np.outer(np.abs(A).max(1), np.abs(B).max(1)) + 2.0 ** -50
+    assert (np.abs(_host(D)[:, :J] - (A[:, pad:] @ B[:, pad:].T + 3.0)) <= bound).all()
+    assert bool((D[:, J:] == 3.0).all())
