@@ -16,7 +16,7 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libnm.so")
 SOURCES = ["kernels.cu", "assemble.cu", "solver.cu", "api.cu", "static_scratch.cu", "mass_tma.cu", "ozaki_gemm.cu", "selfgrav.cu",
-           "kron_cluster.cu", "rows.cu"]
+           "kron_cluster.cu", "rows.cu", "df_rows.cu"]
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 
 

@@ -262,7 +262,6 @@ int nm_set_option(nm_problem* P, const char* key, int64_t value) {
     if (std::string(key) == "df_threads") {
         if (value != 32 && value != 64 && value != 128 && value != 256)
             return fail(NM_EINVAL, "df_threads must be 32, 64, 128 or 256");
-        P->df_threads = (int)value;
         return NM_OK;
     }
     if (std::string(key) == "chunk") {

@@ -987,39 +987,46 @@ __global__ void lo_part_kernel(int64_t n, const double* v, const float* hi, floa
         lo[t] = __double2float_rn(v[t] - (double)hi[t]);
 }
 
-int ensure_f32(nm_problem* P, cudaStream_t s);
+static int to_f32(DevCSR& A, cudaStream_t s) {
+    if (A.nnz == 0 || A.val32.p) return NM_OK;
+    const int64_t cnt = A.nnz * A.rb * A.cb;
+    NM_TRY(A.val32.alloc(cnt * sizeof(float)));
+    return launch_d2f(cnt, A.val.as<double>(), A.val32.as<float>(), s);
+}
 
-// Low float parts of the matrix values for the double-float kernels.
-int ensure_df(nm_problem* P, cudaStream_t s) {
-    NM_TRY(ensure_f32(P, s));
-    for (DevCSR* A : {&P->AG, &P->Mr, &P->Pn}) {
-        if (A->nnz == 0 || A->vlo32.p) continue;
-        const int64_t cnt = A->nnz * A->rb * A->cb;
-        NM_TRY(A->vlo32.alloc(cnt * sizeof(float)));
-        lo_part_kernel<<<(unsigned)std::min<int64_t>((cnt + 255) / 256, 4864), 256, 0, s>>>(
-            cnt, A->val.as<double>(), A->val32.as<float>(), A->vlo32.as<float>());
-        count_launch();
-        NM_CUDA(cudaGetLastError());
+// What the float semi-iterations of the mixed form need: float values and
+// row clusters of the mass and pressure matrices (created on first use).
+int ensure_mixed(nm_problem* P, cudaStream_t s) {
+    for (DevCSR* A : {&P->Mr, &P->Pn}) {
+        NM_TRY(to_f32(*A, s));
+        NM_TRY(build_clusters(*A, s));
     }
     return NM_OK;
 }
 
-// Float copies of the matrix values (created on first FP32 use).
+// What its double-float kernels need besides: the low parts of those values
+// and the records of A_G.
+int ensure_df(nm_problem* P, cudaStream_t s) {
+    NM_TRY(ensure_mixed(P, s));
+    for (DevCSR* A : {&P->Mr, &P->Pn}) {
+        if (A->nnz == 0 || A->vlo32.p) continue;
+        NM_TRY(A->vlo32.alloc(A->nnz * sizeof(float)));
+        lo_part_kernel<<<(unsigned)std::min<int64_t>((A->nnz + 255) / 256, 4864), 256, 0, s>>>(
+            A->nnz, A->val.as<double>(), A->val32.as<float>(), A->vlo32.as<float>());
+        count_launch();
+        NM_CUDA(cudaGetLastError());
+    }
+    if (P->AG.nnz > 0 && !P->AG.rec.p) {
+        NM_TRY(P->AG.rec.alloc(P->AG.nnz * 5 * sizeof(float4)));
+        NM_TRY(launch_df_records(P->AG.nnz, P->AG.val.as<double>(), P->AG.rec.as<float4>(), s));
+    }
+    return NM_OK;
+}
+
+// Float copies of all matrix values (created on first FP32 use).
 int ensure_f32(nm_problem* P, cudaStream_t s) {
-    auto conv = [&](DevCSR& A) -> int {
-        if (A.nnz == 0 || A.val32.p) return NM_OK;
-        const int64_t cnt = A.nnz * A.rb * A.cb;
-        NM_TRY(A.val32.alloc(cnt * sizeof(float)));
-        NM_TRY(launch_d2f(cnt, A.val.as<double>(), A.val32.as<float>(), s));
-        return NM_OK;
-    };
-    NM_TRY(conv(P->AG));
-    NM_TRY(conv(P->Mr));
-    NM_TRY(conv(P->Pn));
-    NM_TRY(conv(P->EG));
-    NM_TRY(conv(P->EGt));
-    NM_TRY(build_clusters(P->Mr, s));
-    if (P->info.Np > 0) NM_TRY(build_clusters(P->Pn, s));
+    NM_TRY(ensure_mixed(P, s));
+    for (DevCSR* A : {&P->AG, &P->EG, &P->EGt}) NM_TRY(to_f32(*A, s));
     return NM_OK;
 }
 

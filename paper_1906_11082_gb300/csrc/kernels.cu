@@ -16,6 +16,7 @@
 #include <type_traits>
 
 #include "nm_internal.h"
+#include "df_convert.cuh"
 
 namespace nm {
 
@@ -723,26 +724,30 @@ __global__ void convert_kernel(int64_t rows, int b, const Tin* X, int64_t ldx, T
     }
 }
 
-// w32 = float(W) and the first semi-iteration step x1 = inv_theta D^-1 w32
-// in one pass (the same float expression as dscale_kernel).
+// w32 = float(W), its low part wl = float(W - w32) and the first
+// semi-iteration step x1 = inv_theta D^-1 w32 in one pass (the same float
+// expression as dscale_kernel).
 __global__ void convert_x1_kernel(int R, int64_t nodes, int b, int bv, const double* W, int64_t ldw, float* w32,
-                                  float inv_theta, const float* dinv, float* x1) {
+                                  float* wl, float inv_theta, const float* dinv, float* x1) {
     const int64_t total = (int64_t)R * nodes * b;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
          t += (int64_t)gridDim.x * blockDim.x) {
         const int64_t r = t / b;
         const int c = (int)(t - r * b);
-        const float w = c < bv ? (float)W[r * ldw + c] : 0.f;
+        const double d = c < bv ? W[r * ldw + c] : 0.0;
+        float w, lo;
+        split_pair(d, w, lo);
         w32[t] = w;
+        if (wl) wl[t] = lo;
         if (x1) x1[t] = inv_theta * dinv[r / R] * w;
     }
 }
 
-int launch_convert_x1(int R, int64_t nodes, int b, int bv, const double* W, int64_t ldw, float* w32, float inv_theta,
-                      const float* dinv, float* x1, cudaStream_t s) {
+int launch_convert_x1(int R, int64_t nodes, int b, int bv, const double* W, int64_t ldw, float* w32, float* wl,
+                      float inv_theta, const float* dinv, float* x1, cudaStream_t s) {
     const int64_t total = (int64_t)R * nodes * b;
     if (total == 0) return NM_OK;
-    convert_x1_kernel<<<grid_for(total), kThreads, 0, s>>>(R, nodes, b, bv, W, ldw, w32, inv_theta, dinv, x1);
+    convert_x1_kernel<<<grid_for(total), kThreads, 0, s>>>(R, nodes, b, bv, W, ldw, w32, wl, inv_theta, dinv, x1);
     count_launch();
     NM_CUDA(cudaGetLastError());
     return NM_OK;
@@ -961,7 +966,7 @@ __global__ void __launch_bounds__(kThreads) combine_kernel(const CombineArgs a) 
         load_n<N>(a.e32 + ix, e);
         double v[N];
 #pragma unroll
-        for (int j = 0; j < N; ++j) v[j] = (double)x[j] + (double)e[j];
+        for (int j = 0; j < N; ++j) v[j] = widen(x[j]) + widen(e[j]);
         if (!a.Tn) {
             store_n<N>(a.out + it, v);
             continue;
@@ -977,10 +982,7 @@ __global__ void __launch_bounds__(kThreads) combine_kernel(const CombineArgs a) 
         if (a.Th) {   // exact float pair of tn for the next double-float K_eff SpMM
             const int64_t ih = (int64_t)i * a.ldh + cg;
 #pragma unroll
-            for (int j = 0; j < N; ++j) {
-                x[j] = __double2float_rn(v[j]);
-                e[j] = __double2float_rn(v[j] - (double)x[j]);
-            }
+            for (int j = 0; j < N; ++j) split_pair(v[j], x[j], e[j]);
             store_n<N>(a.Th + ih, x);
             store_n<N>(a.Tl + ih, e);
         }
@@ -1060,288 +1062,16 @@ int launch_combine(const CombineArgs& a, cudaStream_t s) {
 }
 
 // ----------------------------------------------------------------- double-float
-// sh + sl += (ah + al)(xh + xl) to ~2^-48: TwoProduct of the leading terms by
-// FMA, the cross terms by FMA, TwoSum into the leading accumulator and a
-// FastTwoSum renormalisation. The _rn intrinsics keep the compiler from
-// contracting or reassociating the error-free transformations.
-__device__ __forceinline__ void df_fma(float& sh, float& sl, float ah, float al, float xh, float xl) {
-    const float p = __fmul_rn(ah, xh);
-    const float e = __fmaf_rn(ah, xh, -p);
-    const float t = __fmaf_rn(ah, xl, __fmaf_rn(al, xh, e));
-    const float s = __fadd_rn(sh, p);
-    const float bp = __fadd_rn(s, -sh);
-    const float err = __fadd_rn(__fadd_rn(sh, -__fadd_rn(s, -bp)), __fadd_rn(p, -bp));
-    const float lo = __fadd_rn(__fadd_rn(sl, err), t);
-    sh = __fadd_rn(s, lo);
-    sl = __fadd_rn(lo, -__fadd_rn(sh, -s));
-}
-
 __global__ void split_kernel(int64_t rows, int b, int ldh, const double* X, int64_t ldx, float* Xh, float* Xl) {
     const int64_t total = rows * ldh;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
          t += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i = t / ldh;
         const int c = (int)(t - i * ldh);
-        const double x = c < b ? X[i * ldx + c] : 0.0;
-        const float h = __double2float_rn(x);
+        float h, l;
+        split_pair(c < b ? X[i * ldx + c] : 0.0, h, l);
         Xh[t] = h;
-        Xl[t] = __double2float_rn(x - (double)h);
-    }
-}
-
-template <int CPT>
-__global__ void __launch_bounds__(kThreads) bsr33_df_kernel(const Bsr33DfArgs a, int tpr_shift) {
-    const int tpr = 1 << tpr_shift;
-    const int lane = threadIdx.x & (tpr - 1);
-    const int64_t row = (int64_t)blockIdx.x * (kThreads >> tpr_shift) + (threadIdx.x >> tpr_shift);
-    if (row >= a.nrows) return;
-    float sh[CPT][3], sl[CPT][3];
-#pragma unroll
-    for (int q = 0; q < CPT; ++q)
-#pragma unroll
-        for (int m = 0; m < 3; ++m) sh[q][m] = sl[q][m] = 0.f;
-    const int e0 = __ldg(a.rowptr + row), e1 = __ldg(a.rowptr + row + 1);
-    for (int e = e0; e < e1; ++e) {
-        const int64_t j = __ldg(a.col + e);
-        float kh[9], kl[9];
-#pragma unroll
-        for (int t = 0; t < 9; ++t) {
-            kh[t] = __ldg(a.vh + 9 * (int64_t)e + t);
-            kl[t] = __ldg(a.vl + 9 * (int64_t)e + t);
-        }
-        const int64_t base = 3 * j * a.ldx;
-#pragma unroll
-        for (int q = 0; q < CPT; ++q) {
-            const int c = lane + q * tpr;
-            if (c < a.b) {
-                float xh[3], xl[3];
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    xh[k] = __ldg(a.Xh + base + k * a.ldx + c);
-                    xl[k] = __ldg(a.Xl + base + k * a.ldx + c);
-                }
-#pragma unroll
-                for (int m = 0; m < 3; ++m)
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) df_fma(sh[q][m], sl[q][m], kh[3 * m + k], kl[3 * m + k], xh[k], xl[k]);
-            }
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < CPT; ++q) {
-        const int c = lane + q * tpr;
-        if (c >= a.b) continue;
-        double acc[3];
-#pragma unroll
-        for (int m = 0; m < 3; ++m) acc[m] = (double)sh[q][m] + (double)sl[q][m];
-        if (a.e_rowptr) {
-            const int f0 = __ldg(a.e_rowptr + row), f1 = __ldg(a.e_rowptr + row + 1);
-            for (int e = f0; e < f1; ++e) {
-                const int64_t p = __ldg(a.e_col + e);
-                const double sv = __ldg(a.S + p * a.lds + c);
-#pragma unroll
-                for (int m = 0; m < 3; ++m) acc[m] += __ldg(a.e_val + 3 * (int64_t)e + m) * sv;
-            }
-        }
-#pragma unroll
-        for (int m = 0; m < 3; ++m) a.W[(3 * row + m) * a.ldw + c] = acc[m];
-    }
-}
-
-template <int R, int CPT>
-__global__ void __launch_bounds__(kThreads) resid_df_kernel(int64_t nodes, const int* __restrict__ rowptr,
-                                                            const int* __restrict__ col, const float* __restrict__ vh,
-                                                            const float* __restrict__ vl, const double* __restrict__ W,
-                                                            int64_t ldw, const float* __restrict__ x, float* r, int b,
-                                                            int bv, int tpr_shift) {
-    const int tpr = 1 << tpr_shift;
-    const int lane = threadIdx.x & (tpr - 1);
-    const int64_t row = (int64_t)blockIdx.x * (kThreads >> tpr_shift) + (threadIdx.x >> tpr_shift);
-    if (row >= nodes) return;
-    float sh[CPT][R], sl[CPT][R];
-#pragma unroll
-    for (int q = 0; q < CPT; ++q)
-#pragma unroll
-        for (int k = 0; k < R; ++k) sh[q][k] = sl[q][k] = 0.f;
-    const int e0 = __ldg(rowptr + row), e1 = __ldg(rowptr + row + 1);
-    for (int e = e0; e < e1; ++e) {
-        const int64_t j = __ldg(col + e);
-        const float mh = __ldg(vh + e), ml = __ldg(vl + e);
-        const float* xj = x + (int64_t)R * j * b;
-#pragma unroll
-        for (int q = 0; q < CPT; ++q) {
-            const int c = lane + q * tpr;
-            if (c < b) {
-#pragma unroll
-                for (int k = 0; k < R; ++k) df_fma(sh[q][k], sl[q][k], mh, ml, __ldg(xj + k * b + c), 0.f);
-            }
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < CPT; ++q) {
-        const int c = lane + q * tpr;
-        if (c >= b) continue;
-#pragma unroll
-        for (int k = 0; k < R; ++k) {
-            const int64_t rr = R * row + k;
-            r[rr * b + c] = (float)(((c < bv ? W[rr * ldw + c] : 0.0) - (double)sh[q][k]) - (double)sl[q][k]);
-        }
-    }
-}
-
-// Dot2-style double-float accumulation (Ogita, Rump and Oishi): the
-// rounding error of each product (exact via FMA), the first-order terms of
-// the operands' low parts and the TwoSum error of each addition are
-// collected in sl; sh carries the running float sum. sl stays ~n ulp(sh),
-// so it needs no renormalisation until the final (double) sh + sl.
-__device__ __forceinline__ void df_acc(float& sh, float& sl, float ah, float al, float xh, float xl) {
-    const float p = __fmul_rn(ah, xh);
-    const float e = __fmaf_rn(ah, xh, -p);
-    const float t = __fmaf_rn(ah, xl, __fmaf_rn(al, xh, e));
-    const float s = __fadd_rn(sh, p);
-    const float bp = __fadd_rn(s, -sh);
-    const float err = __fadd_rn(__fadd_rn(sh, -__fadd_rn(s, -bp)), __fadd_rn(p, -bp));
-    sh = s;
-    sl = __fadd_rn(sl, __fadd_rn(err, t));
-}
-
-// (sh, sl) += (h2, l2) for two Dot2 accumulators.
-__device__ __forceinline__ void df_merge(float& sh, float& sl, float h2, float l2) {
-    const float s = __fadd_rn(sh, h2);
-    const float bp = __fadd_rn(s, -sh);
-    const float err = __fadd_rn(__fadd_rn(sh, -__fadd_rn(s, -bp)), __fadd_rn(h2, -bp));
-    sh = s;
-    sl = __fadd_rn(sl, __fadd_rn(err, l2));
-}
-
-// Butterfly-combine the four lane groups' accumulators (lanes q, q + 8,
-// q + 16, q + 24 hold partial sums of the same four columns).
-template <int N>
-__device__ __forceinline__ void df_group_reduce(float (&sh)[N], float (&sl)[N]) {
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-#pragma unroll
-        for (int m = 8; m <= 16; m *= 2) {
-            const float h2 = __shfl_xor_sync(0xffffffffu, sh[i], m);
-            const float l2 = __shfl_xor_sync(0xffffffffu, sl[i], m);
-            df_merge(sh[i], sl[i], h2, l2);
-        }
-    }
-}
-
-// W = A X (+ E S) in double-float for blocks exactly 32 wide with the split
-// operand stored densely (ld 32): one warp per 3x3-block row, four groups
-// of eight lanes taking every fourth stored block, lane q of a group
-// holding columns 4q..4q+3 of the three output components and reading the
-// neighbour's (hi, lo) records with 16-byte loads. After the groups are
-// combined, group m < 3 writes output component m (and adds the pressure
-// coupling in double, as the generic kernel does).
-template <int NT>
-__global__ void __launch_bounds__(NT, 1024 / NT) bsr33_df_v4_kernel(const Bsr33DfArgs a) {
-    const int lane = threadIdx.x & 31;
-    const int g = lane >> 3, q = lane & 7;
-    const int64_t row = (int64_t)blockIdx.x * (NT / 32) + (threadIdx.x >> 5);
-    if (row >= a.nrows) return;
-    float sh[12], sl[12];
-#pragma unroll
-    for (int i = 0; i < 12; ++i) sh[i] = sl[i] = 0.f;
-    const int e0 = __ldg(a.rowptr + row), e1 = __ldg(a.rowptr + row + 1);
-    const float4* xh4 = reinterpret_cast<const float4*>(a.Xh) + q;
-    const float4* xl4 = reinterpret_cast<const float4*>(a.Xl) + q;
-    for (int e = e0 + g; e < e1; e += 4) {
-        const int64_t j = __ldg(a.col + e);
-        const float* kh = a.vh + 9 * (int64_t)e;
-        const float* kl = a.vl + 9 * (int64_t)e;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const float4 xh = __ldg(xh4 + j * 24 + 8 * k);
-            const float4 xl = __ldg(xl4 + j * 24 + 8 * k);
-#pragma unroll
-            for (int m = 0; m < 3; ++m) {
-                const float ah = __ldg(kh + 3 * m + k), al = __ldg(kl + 3 * m + k);
-                df_acc(sh[4 * m + 0], sl[4 * m + 0], ah, al, xh.x, xl.x);
-                df_acc(sh[4 * m + 1], sl[4 * m + 1], ah, al, xh.y, xl.y);
-                df_acc(sh[4 * m + 2], sl[4 * m + 2], ah, al, xh.z, xl.z);
-                df_acc(sh[4 * m + 3], sl[4 * m + 3], ah, al, xh.w, xl.w);
-            }
-        }
-    }
-    df_group_reduce<12>(sh, sl);
-    if (g >= 3) return;
-    const int m = g;
-    double acc[4];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const float h = m == 0 ? sh[c] : (m == 1 ? sh[4 + c] : sh[8 + c]);
-        const float l = m == 0 ? sl[c] : (m == 1 ? sl[4 + c] : sl[8 + c]);
-        acc[c] = (double)h + (double)l;
-    }
-    if (a.e_rowptr) {
-        const int f0 = __ldg(a.e_rowptr + row), f1 = __ldg(a.e_rowptr + row + 1);
-        for (int f = f0; f < f1; ++f) {
-            const int64_t p = __ldg(a.e_col + f);
-            const double ev = __ldg(a.e_val + 3 * (int64_t)f + m);
-            const double* sp = a.S + p * a.lds + 4 * q;
-#pragma unroll
-            for (int c = 0; c < 4; ++c) acc[c] += ev * __ldg(sp + c);
-        }
-    }
-    double* wp = a.W + (3 * row + m) * a.ldw + 4 * q;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) wp[c] = acc[c];
-}
-
-// r32 = float(W - (A (x) I_R) x32) for blocks exactly 32 wide (x32 and r32
-// dense, ld 32), with the lane-group layout of bsr33_df_v4_kernel.
-template <int R, int NT>
-__global__ void __launch_bounds__(NT, 1024 / NT) resid_df_v4_kernel(int64_t nodes, const int* __restrict__ rowptr,
-                                                                  const int* __restrict__ col,
-                                                                  const float* __restrict__ vh,
-                                                                  const float* __restrict__ vl,
-                                                                  const double* __restrict__ W, int64_t ldw,
-                                                                  const float* __restrict__ x, float* r,
-                                                                  const float* __restrict__ dinv, float inv_theta,
-                                                                  float* x1) {
-    const int lane = threadIdx.x & 31;
-    const int g = lane >> 3, q = lane & 7;
-    const int64_t row = (int64_t)blockIdx.x * (NT / 32) + (threadIdx.x >> 5);
-    if (row >= nodes) return;
-    float sh[4 * R], sl[4 * R];
-#pragma unroll
-    for (int i = 0; i < 4 * R; ++i) sh[i] = sl[i] = 0.f;
-    const int e0 = __ldg(rowptr + row), e1 = __ldg(rowptr + row + 1);
-    const float4* x4 = reinterpret_cast<const float4*>(x) + q;
-    for (int e = e0 + g; e < e1; e += 4) {
-        const int64_t j = __ldg(col + e);
-        const float mh = __ldg(vh + e), ml = __ldg(vl + e);
-#pragma unroll
-        for (int k = 0; k < R; ++k) {
-            const float4 xv = __ldg(x4 + j * (8 * R) + 8 * k);
-            df_acc(sh[4 * k + 0], sl[4 * k + 0], mh, ml, xv.x, 0.f);
-            df_acc(sh[4 * k + 1], sl[4 * k + 1], mh, ml, xv.y, 0.f);
-            df_acc(sh[4 * k + 2], sl[4 * k + 2], mh, ml, xv.z, 0.f);
-            df_acc(sh[4 * k + 3], sl[4 * k + 3], mh, ml, xv.w, 0.f);
-        }
-    }
-    df_group_reduce<4 * R>(sh, sl);
-    if (g >= R) return;
-    const int k = g;
-    const int64_t rr = R * row + k;
-    const double* wp = W + rr * ldw + 4 * q;
-    float out[4];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        float h = sh[c], l = sl[c];
-        if (R == 3) {
-            h = k == 0 ? sh[c] : (k == 1 ? sh[4 + c] : sh[8 + c]);
-            l = k == 0 ? sl[c] : (k == 1 ? sl[4 + c] : sl[8 + c]);
-        }
-        out[c] = (float)((wp[c] - (double)h) - (double)l);
-    }
-    reinterpret_cast<float4*>(r + rr * 32)[q] = make_float4(out[0], out[1], out[2], out[3]);
-    if (x1) {   // first semi-iteration step on r, as dscale_kernel computes it
-        const float d = inv_theta * dinv[row];
-        reinterpret_cast<float4*>(x1 + rr * 32)[q] = make_float4(d * out[0], d * out[1], d * out[2], d * out[3]);
+        Xl[t] = l;
     }
 }
 
@@ -1350,84 +1080,6 @@ int launch_split(int64_t rows, int b, int ldh, const double* X, int64_t ldx, flo
     split_kernel<<<grid_for(rows * ldh), kThreads, 0, s>>>(rows, b, ldh, X, ldx, Xh, Xl);
     count_launch();
     NM_CUDA(cudaGetLastError());
-    return NM_OK;
-}
-
-int launch_bsr33_df(const Bsr33DfArgs& a, cudaStream_t s) {
-    if (a.b < 1 || a.b > 64) return fail(NM_EINVAL, "block width must be in 1..64");
-    if (a.vec && a.b == 32 && a.ldx == 32 && (((uintptr_t)a.Xh | (uintptr_t)a.Xl) & 15) == 0) {
-        const int nt = a.nt;
-        const int64_t grid = (a.nrows + nt / 32 - 1) / (nt / 32);
-        if (grid == 0) return NM_OK;
-        switch (nt) {
-            case 32: bsr33_df_v4_kernel<32><<<(unsigned)grid, 32, 0, s>>>(a); break;
-            case 64: bsr33_df_v4_kernel<64><<<(unsigned)grid, 64, 0, s>>>(a); break;
-            case 128: bsr33_df_v4_kernel<128><<<(unsigned)grid, 128, 0, s>>>(a); break;
-            default: bsr33_df_v4_kernel<256><<<(unsigned)grid, 256, 0, s>>>(a); break;
-        }
-        count_launch();
-        NM_CUDA(cudaGetLastError());
-        return NM_OK;
-    }
-    const int shift = tpr_shift_for(a.b);
-    const int cpt = (a.b + (1 << shift) - 1) >> shift;
-    const int64_t grid = (a.nrows + (kThreads >> shift) - 1) / (kThreads >> shift);
-    if (grid == 0) return NM_OK;
-    if (cpt == 1)
-        bsr33_df_kernel<1><<<(unsigned)grid, kThreads, 0, s>>>(a, shift);
-    else
-        bsr33_df_kernel<2><<<(unsigned)grid, kThreads, 0, s>>>(a, shift);
-    count_launch();
-    NM_CUDA(cudaGetLastError());
-    return NM_OK;
-}
-
-int launch_resid_df(int R, int64_t nodes, const int* rowptr, const int* col, const float* vh, const float* vl,
-                    const double* W, int64_t ldw, const float* x32, float* r32, int b, int bv, cudaStream_t s, int vec,
-                    int nt, const float* dinv, float inv_theta, float* x1) {
-    if (b < 1 || b > 64) return fail(NM_EINVAL, "block width must be in 1..64");
-    if (vec && b == 32 && bv == 32 && (((uintptr_t)x32 | (uintptr_t)r32 | (uintptr_t)x1) & 15) == 0) {
-        if (nt != 32 && nt != 64 && nt != 128) nt = 256;
-        const int64_t grid = (nodes + nt / 32 - 1) / (nt / 32);
-        if (grid == 0) return NM_OK;
-#define NM_RESID_V4(RR, NN) \
-    resid_df_v4_kernel<RR, NN><<<(unsigned)grid, NN, 0, s>>>(nodes, rowptr, col, vh, vl, W, ldw, x32, r32, dinv, \
-                                                            inv_theta, x1)
-        if (R == 3) {
-            switch (nt) {
-                case 32: NM_RESID_V4(3, 32); break;
-                case 64: NM_RESID_V4(3, 64); break;
-                case 128: NM_RESID_V4(3, 128); break;
-                default: NM_RESID_V4(3, 256); break;
-            }
-        } else {
-            switch (nt) {
-                case 32: NM_RESID_V4(1, 32); break;
-                case 64: NM_RESID_V4(1, 64); break;
-                case 128: NM_RESID_V4(1, 128); break;
-                default: NM_RESID_V4(1, 256); break;
-            }
-        }
-#undef NM_RESID_V4
-        count_launch();
-        NM_CUDA(cudaGetLastError());
-        return NM_OK;
-    }
-    const int shift = tpr_shift_for(b);
-    const int cpt = (b + (1 << shift) - 1) >> shift;
-    const int64_t grid = (nodes + (kThreads >> shift) - 1) / (kThreads >> shift);
-    if (grid == 0) return NM_OK;
-    if (R == 3 && cpt == 1)
-        resid_df_kernel<3, 1><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, vh, vl, W, ldw, x32, r32, b, bv, shift);
-    else if (R == 3)
-        resid_df_kernel<3, 2><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, vh, vl, W, ldw, x32, r32, b, bv, shift);
-    else if (cpt == 1)
-        resid_df_kernel<1, 1><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, vh, vl, W, ldw, x32, r32, b, bv, shift);
-    else
-        resid_df_kernel<1, 2><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, vh, vl, W, ldw, x32, r32, b, bv, shift);
-    count_launch();
-    NM_CUDA(cudaGetLastError());
-    if (x1) return launch_dscale<float>(R, nodes, b, inv_theta, dinv, r32, b, x1, b, s);
     return NM_OK;
 }
 

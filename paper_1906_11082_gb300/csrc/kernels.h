@@ -228,14 +228,14 @@ int launch_bsr31_add(int nrows, const int* rowptr, const int* col, const double*
 // Split a double block into exact float pairs (hi = fl(x), lo = fl(x - hi)),
 // ldh columns wide, those from b on zero.
 int launch_split(int64_t rows, int b, int ldh, const double* X, int64_t ldx, float* Xh, float* Xl, cudaStream_t s);
-// W = A X + E S with A's 3x3 blocks as (hi, lo) floats and X as (hi, lo)
-// float blocks (ld ldx), double-float sums; the optional E S part in double.
+// W = A X + E S with A's 3x3 blocks as 80-byte records (nine high, nine low
+// parts, two zeros) and X as (hi, lo) float blocks, double-float sums; the
+// optional E S part in double. X is ldx = ng bg columns wide (cluster_groups).
 struct Bsr33DfArgs {
     int nrows = 0;
-    const int* rowptr = nullptr;
+    const int4* desc = nullptr;
     const int* col = nullptr;
-    const float* vh = nullptr;
-    const float* vl = nullptr;
+    const float4* vhl = nullptr;
     const float* Xh = nullptr;
     const float* Xl = nullptr;
     int b = 0;
@@ -247,23 +247,33 @@ struct Bsr33DfArgs {
     int64_t lds = 0;
     double* W = nullptr;
     int64_t ldw = 0;
-    int vec = 1;   // b = 32 with 16-byte aligned operands: lane-group kernel
-    int nt = 256;  // its CTA size (32, 64, 128, 256)
 };
 int launch_bsr33_df(const Bsr33DfArgs& a, cudaStream_t s);
-// r32 = float(W - (A (x) I_R) x32) with A as (hi, lo) floats, double-float
-// sums; x32 and r32 dense (ld b); W holds the first bv of the b columns.
-// vec: lane-group kernel when b = bv = 32.
-int launch_resid_df(int R, int64_t nodes, const int* rowptr, const int* col, const float* vh, const float* vl,
-                    const double* W, int64_t ldw, const float* x32, float* r32, int b, int bv, cudaStream_t s,
-                    int vec = 1, int nt = 256, const float* dinv = nullptr, float inv_theta = 0.f,
-                    float* x1 = nullptr);
-// With x1 != nullptr also writes the first semi-iteration step on r32,
-// x1 = inv_theta D^-1 r32 (dinv per node, ld b).
-// w32 = float(W) and, with x1 != nullptr, x1 = inv_theta D^-1 w32 in one pass
-// (w32, x1 dense, b wide; W holds the first bv columns, the others are zero).
-int launch_convert_x1(int R, int64_t nodes, int b, int bv, const double* W, int64_t ldw, float* w32, float inv_theta,
-                      const float* dinv, float* x1, cudaStream_t s);
+// The records of n blocks.
+int launch_df_records(int64_t n, const double* val, float4* out, cudaStream_t s);
+// r = w - (A (x) I_R) x with w and A as (hi, lo) floats, double-float sums;
+// all blocks dense, b columns (a multiple of four, at most 32); r may be wh.
+// With x1 also the first semi-iteration step on r, x1 = inv_theta D^-1 r.
+struct ResidDfArgs {
+    int nrows = 0;
+    const int4* desc = nullptr;
+    const int* col = nullptr;
+    const float* vh = nullptr;
+    const float* vl = nullptr;
+    const float* wh = nullptr;
+    const float* wl = nullptr;
+    const float* x = nullptr;
+    float* r = nullptr;
+    const float* dinv = nullptr;
+    float inv_theta = 0.f;
+    float* x1 = nullptr;
+};
+int launch_resid_df(int R, const ResidDfArgs& a, int b, cudaStream_t s);
+// w32 = float(W) and, where given, wl = float(W - w32) and x1 = inv_theta D^-1
+// w32 in one pass (w32, wl, x1 dense, b wide; W holds the first bv columns, the
+// others are zero).
+int launch_convert_x1(int R, int64_t nodes, int b, int bv, const double* W, int64_t ldw, float* w32, float* wl,
+                      float inv_theta, const float* dinv, float* x1, cudaStream_t s);
 
 // Y[i, c] = alpha * X[i, c] (rows x b, row-major with leading dims).
 template <typename T>

@@ -74,7 +74,8 @@ struct DevCSR {
     DevBuf col;      // int32 [nnz]
     DevBuf val;      // double [nnz * rb * cb]
     DevBuf val32;    // float  [nnz * rb * cb] (on demand): fl(val), the high part
-    DevBuf vlo32;    // float  [nnz * rb * cb] (on demand): fl(val - fl(val)), the low part
+    DevBuf vlo32;    // float  [nnz * rb * cb] (on demand): fl(val - fl(val)), the low part (scalar matrices)
+    DevBuf rec;      // float4 [5 nnz] (on demand): 3x3 blocks as high and low parts (df_rows.cu)
     DevBuf desc;     // int4 [nrows]: row, first entry, end, in launch order (rows.cu)
     DevBuf dinv;     // inverse diagonal (scalar square matrices only), double
     DevBuf dinv32;
@@ -199,7 +200,6 @@ struct nm_problem {
     int use_tma = 0;      // shared-memory staged tiles for the float b = 32 mass steps (option "tma")
     int vec_threads = 32;   // their CTA size (3-component rows)
     int vec_threads_p = 128;  // ... and for the 1-component pressure rows
-    int df_threads = 32;    // CTA size of the lane-group double-float kernels
     int use_chunk = 0;    // threads per CTA of the chunked row schedule, 0 = off
     nm::DevBuf sched;   // int [nreg] region counters
     int nreg = 0;

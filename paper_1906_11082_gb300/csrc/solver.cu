@@ -19,6 +19,7 @@
 namespace nm {
 
 int ensure_f32(nm_problem* P, cudaStream_t s);
+int ensure_mixed(nm_problem* P, cudaStream_t s);
 int ensure_df(nm_problem* P, cudaStream_t s);
 template <typename T>
 int filter_apply_t(nm_problem* P, const nm_filter* f, const T* Y, int64_t ldy, T* Z, int64_t ldz, int b, cudaStream_t s);
@@ -401,9 +402,7 @@ struct MixScratch {
 
 static int get_mix_scratch(nm_problem* P, int b, MixScratch& S) {
     const int64_t n = P->info.n, Np = P->info.Np;
-    S.ng = 1;
-    S.bg = b;
-    if (use_clusters(P->Mr, P) && !(b == 32 && P->use_tma)) cluster_groups(b, &S.ng, &S.bg);
+    cluster_groups(b, &S.ng, &S.bg);
     S.bp = S.ng * S.bg;
     // 16-byte aligned parts
     const int64_t nd = (n * b + 1) / 2 * 2, pd = (Np * b + 1) / 2 * 2, ng = (n * S.bg + 3) / 4 * 4, np = (n * S.bp + 3) / 4 * 4;
@@ -487,13 +486,26 @@ static int mixed_solve(nm_problem* P, const DevCSR& A, int R, int bv, int k, con
     // k >= 2: the float conversion of W and the double-float residual also
     // write the first semi-iteration step, so cheb32 starts at step 2
     const bool fuse = k >= 2;
-    NM_TRY(launch_convert_x1(R, A.nrows, b, bv, W, ldw, S.w32, it, A.dinv32.as<float>(), fuse ? S.xa : nullptr, s));
+    // S.es is free until the second solve writes it: the low part of W
+    float* wl = df ? S.es : nullptr;
+    NM_TRY(launch_convert_x1(R, A.nrows, b, bv, W, ldw, S.w32, wl, it, A.dinv32.as<float>(), fuse ? S.xa : nullptr, s));
     NM_TRY(cheb32(P, A, R, b, k, kMassLo, kMassHi, S.w32, S.xa, S.xb, S.xs, s, fuse));
     bool x1 = false;
     if (df) {
-        NM_TRY(launch_resid_df(R, A.nrows, A.rowptr.as<int>(), A.col.as<int>(), A.val32.as<float>(),
-                               A.vlo32.as<float>(), W, ldw, S.xs, S.w32, b, bv, s, P->use_vec, P->df_threads,
-                               A.dinv32.as<float>(), it, fuse ? S.xa : nullptr));
+        ResidDfArgs r;
+        r.nrows = (int)A.nrows;
+        r.desc = A.desc.as<int4>();
+        r.col = A.col.as<int>();
+        r.vh = A.val32.as<float>();
+        r.vl = A.vlo32.as<float>();
+        r.wh = S.w32;
+        r.wl = wl;
+        r.x = S.xs;
+        r.r = S.w32;
+        r.dinv = A.dinv32.as<float>();
+        r.inv_theta = it;
+        r.x1 = fuse ? S.xa : nullptr;
+        NM_TRY(launch_resid_df(R, r, b, s));
         x1 = fuse;
     } else {
         NM_TRY(launch_resid_mixed(R, A.nrows, A.rowptr.as<int>(), A.col.as<int>(), A.val.as<double>(), W, ldw,
@@ -597,18 +609,15 @@ static int apply_K_mixed_core(nm_problem* P, const double* X, int64_t ldx, doubl
         } else {
             Bsr33DfArgs f;
             f.nrows = a.nrows;
-            f.rowptr = a.rowptr;
+            f.desc = a.desc;
             f.col = a.col;
-            f.vh = P->AG.val32.as<float>();
-            f.vl = P->AG.vlo32.as<float>();
+            f.vhl = P->AG.rec.as<float4>();
             f.Xh = S.Th;
             f.Xl = S.Tl;
             f.b = b;
             f.ldx = S.bp;
             f.W = W;
             f.ldw = ldw;
-            f.vec = P->use_vec;
-            f.nt = P->df_threads;
             NM_TRY(launch_bsr33_df(f, s));
         }
         NM_CUDA(cudaStreamWaitEvent(s, P->ev_join, 0));
@@ -617,10 +626,9 @@ static int apply_K_mixed_core(nm_problem* P, const double* X, int64_t ldx, doubl
     if (!df) return launch_bsr33<double>(a, s);
     Bsr33DfArgs f;
     f.nrows = a.nrows;
-    f.rowptr = a.rowptr;
+    f.desc = a.desc;
     f.col = a.col;
-    f.vh = P->AG.val32.as<float>();
-    f.vl = P->AG.vlo32.as<float>();
+    f.vhl = P->AG.rec.as<float4>();
     f.Xh = S.Th;
     f.Xl = S.Tl;
     f.b = b;
@@ -632,8 +640,6 @@ static int apply_K_mixed_core(nm_problem* P, const double* X, int64_t ldx, doubl
     f.lds = a.lds;
     f.W = W;
     f.ldw = ldw;
-    f.vec = P->use_vec;
-    f.nt = P->df_threads;
     return launch_bsr33_df(f, s);
 }
 
@@ -644,7 +650,7 @@ static int filter_apply_mixed(nm_problem* P, const nm_filter* f, const double* Y
     if (f->k_M < 1 || (P->info.Np > 0 && f->k_P < 1)) return fail(NM_EINVAL, "k_M and k_P must be >= 1");
     if (!(f->e > 0)) return fail(NM_EINVAL, "filter half-width e must be positive");
     if (f->m_lo > 0 || f->m_hi > 0) return fail(NM_EUNSUPPORTED, "mixed mode uses the P2 element bounds");
-    NM_TRY(ensure_f32(P, s));
+    NM_TRY(ensure_mixed(P, s));
     if (P->use_df) NM_TRY(ensure_df(P, s));
     if (b == 32 && P->use_tma) NM_TRY(build_tma_tiles(P->Mr, s));
     const int64_t n = P->info.n;
@@ -789,7 +795,7 @@ int filter_apply_mixed_pub(nm_problem* P, const nm_filter* f, const double* Y, i
 
 int apply_K_mixed_pub(nm_problem* P, const double* X, int64_t ldx, double* Y, int64_t ldy, int b, int k_P,
                       cudaStream_t s) {
-    NM_TRY(ensure_f32(P, s));
+    NM_TRY(ensure_mixed(P, s));
     if (P->use_df) NM_TRY(ensure_df(P, s));
     MixScratch S;
     NM_TRY(get_mix_scratch(P, b, S));
@@ -798,7 +804,7 @@ int apply_K_mixed_pub(nm_problem* P, const double* X, int64_t ldx, double* Y, in
 
 int solve_M_mixed_pub(nm_problem* P, int k_M, const double* W, int64_t ldw, double* X, int64_t ldx, int b,
                       cudaStream_t s) {
-    NM_TRY(ensure_f32(P, s));
+    NM_TRY(ensure_mixed(P, s));
     if (P->use_df) NM_TRY(ensure_df(P, s));
     if (b == 32 && P->use_tma) NM_TRY(build_tma_tiles(P->Mr, s));
     MixScratch S;

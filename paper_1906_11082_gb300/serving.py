@@ -79,11 +79,12 @@ def _batch_sig(opts):
 
 def problem_bytes(info):
     """Device bytes of a resident problem from the library's counts: the
-    FP64 matrices, their float and double-float copies, the reference field
-    and the filter recurrence scratch of a full 64-column batch."""
+    FP64 matrices, their float and double-float copies, the row clusters, the
+    reference field and the filter recurrence scratch of a full 64-column
+    batch."""
     nnz_u, nnz_p, nnz_e = info["nnz_u"], info["nnz_p"], info["nnz_e"]
     n, Np, Nu = info["n"], info["Np"], info["Nu"]
-    mats = nnz_u * (9 * 8 + 4 + 8 + 2 * 9 * 4 + 3 * 4) + nnz_p * (8 + 4 + 3 * 4) + 2 * nnz_e * (3 * 8 + 4)
+    mats = nnz_u * (9 * 8 + 4 + 8 + 80 + 3 * 4 + 12) + nnz_p * (8 + 4 + 3 * 4 + 12) + 2 * nnz_e * (3 * 8 + 4)
     mats += 4 * (Nu + Np) * 8 + 3 * Nu * 8
     scratch = (n * _MAX_COLS) * (3 * 8 + 7 * 4) + Np * _MAX_COLS * 3 * 8
     return int(1.2 * (mats + scratch))

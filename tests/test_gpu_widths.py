@@ -147,3 +147,18 @@ def test_split_products_odd_strides(nm, ctx, I, J, K, pad):
     bound = K * 2.0 ** -50 * np.outer(np.abs(A).max(1), np.abs(B).max(1)) + 2.0 ** -50
     assert (np.abs(_host(D)[:, :J] - (A[:, pad:] @ B[:, pad:].T + 3.0)) <= bound).all()
     assert bool((D[:, J:] == 3.0).all())
+
+
+@pytest.mark.parametrize("b", [1, 5, 12, 16, 20, 24, 28, 32, 33, 48, 64])
+def test_mixed_product_every_width(nm, planet, b):
+    """Double-float K_eff product and residuals at every lane count, padded
+    and two-group widths; fluid rows take E_G S in double. Tolerance as for
+    the refined pressure solve at k = 28."""
+    S, P = planet
+    Xc = np.random.default_rng(b).standard_normal((S.n, b))
+    Xc[::7] *= 1e-30                     # conversions outside their fast range
+    Xc[5] = 0.0
+    Y = torch.empty((S.n, b), dtype=torch.float64, device=DEV)
+    P.apply_K(_dev(to_internal(P, Xc)), Y, k_P=28, prec=nm.NM_MIXED)
+    op = filtlan.Operator(S, k_M=28, k_P=28, refine=True)
+    assert rel_err(to_canonical(P, _host(Y)), op.K(Xc)) <= 1e-11
