@@ -40,33 +40,54 @@ namespace {
 constexpr int kThreads = 64;
 constexpr int kWindow = 64;
 
-// VW consecutive values (16-byte aligned when VW = 2 doubles / 8 when 2 floats)
+// VW consecutive values of a row of which n exist. PAIR: two-value accesses
+// (even widths and strides, aligned operands).
 template <typename T, int VW>
 struct Vec {
     T v[VW];
 };
-template <typename T, int VW>
-__device__ __forceinline__ Vec<T, VW> ld(const T* p) {
+template <typename T>
+struct Pair;
+template <>
+struct Pair<double> {
+    using type = double2;
+};
+template <>
+struct Pair<float> {
+    using type = float2;
+};
+template <bool PAIR, typename T, int VW>
+__device__ __forceinline__ Vec<T, VW> ld(const T* p, int n) {
     Vec<T, VW> r;
-    if constexpr (VW == 1) {
-        r.v[0] = *p;
-    } else if constexpr (sizeof(T) == 8) {
-        const double2 t = *reinterpret_cast<const double2*>(p);
-        r.v[0] = t.x, r.v[1] = t.y;
+    if constexpr (PAIR) {
+        using P = typename Pair<T>::type;
+#pragma unroll
+        for (int i = 0; i < VW; i += 2) {
+            P t;
+            t.x = t.y = T(0);
+            if (i < n) t = *reinterpret_cast<const P*>(p + i);
+            r.v[i] = t.x, r.v[i + 1] = t.y;
+        }
     } else {
-        const float2 t = *reinterpret_cast<const float2*>(p);
-        r.v[0] = t.x, r.v[1] = t.y;
+#pragma unroll
+        for (int i = 0; i < VW; ++i) r.v[i] = i < n ? p[i] : T(0);
     }
     return r;
 }
-template <typename T, int VW>
-__device__ __forceinline__ void st(T* p, const Vec<T, VW>& r) {
-    if constexpr (VW == 1) {
-        *p = r.v[0];
-    } else if constexpr (sizeof(T) == 8) {
-        *reinterpret_cast<double2*>(p) = make_double2(r.v[0], r.v[1]);
+template <bool PAIR, typename T, int VW>
+__device__ __forceinline__ void st(T* p, const Vec<T, VW>& r, int n) {
+    if constexpr (PAIR) {
+        using P = typename Pair<T>::type;
+#pragma unroll
+        for (int i = 0; i < VW; i += 2) {
+            P t;
+            t.x = r.v[i], t.y = r.v[i + 1];
+            if (i < n) *reinterpret_cast<P*>(p + i) = t;
+        }
     } else {
-        *reinterpret_cast<float2*>(p) = make_float2(r.v[0], r.v[1]);
+#pragma unroll
+        for (int i = 0; i < VW; ++i)
+            if (i < n) p[i] = r.v[i];
     }
 }
 template <typename T, int VW>
@@ -136,33 +157,34 @@ struct Scatter {
     }
 };
 
-// Where a lane works: lane q of split sp of row slot `slot`; column c (of
-// VW), valid columns only where on.
+// Where a lane works: split sp of a row, columns c .. c + n - 1 (n = 0: no
+// row). L lanes cover the columns; with splits L is a power of two.
 struct Place {
-    int sp, c;
-    bool on;
+    int sp, c, n;
     int4 d;   // row, first entry, end
 };
 template <int VW, int S>
-__device__ __forceinline__ Place place(const int4* desc, int nrows, int b, int tl_shift) {
+__device__ __forceinline__ Place place(const int4* desc, int nrows, int b, int L) {
     Place p;
-    const int t = blockIdx.x * kThreads + threadIdx.x;
-    const int slot = t >> tl_shift >> (S == 1 ? 0 : S == 2 ? 1 : S == 4 ? 2 : 3);
-    p.sp = (t >> tl_shift) & (S - 1);
-    p.c = VW * ((t & ((1 << tl_shift) - 1)) + (blockIdx.y << tl_shift));
-    p.on = slot < nrows && p.c < b;
-    p.d = __ldg(desc + min(slot, nrows - 1));
-    if (!p.on) p.d.z = p.d.y;   // no entries
+    const int lane = threadIdx.x & 31, lc = L * S, per = 32 / lc;
+    const int cw = lane / lc, rl = lane - cw * lc;
+    p.sp = rl / L;
+    p.c = VW * (rl - p.sp * L + blockIdx.y * L);
+    const int slot = (blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5)) * per + cw;
+    const bool on = cw < per && slot < nrows && p.c < b;
+    p.d = __ldg(desc + (on ? slot : 0));
+    p.n = on ? min(VW, b - p.c) : 0;
+    if (!on) p.c = 0, p.d.z = p.d.y;   // no entries
     return p;
 }
 
 }  // namespace
 
 // ----------------------------------------------------------------- A (x) I_R
-template <typename T, int R, int MODE, int VW, int S, int U>
-__global__ void __launch_bounds__(kThreads) kron_rows_kernel(const KronArgs<T> a, int tl_shift) {
-    const Place p = place<VW, S>(a.desc, a.nrows, a.b, tl_shift);
-    const int c = p.on ? p.c : 0;
+template <typename T, int R, int MODE, int VW, bool PAIR, int S, int U>
+__global__ void __launch_bounds__(kThreads) kron_rows_kernel(const KronArgs<T> a, int L) {
+    const Place p = place<VW, S>(a.desc, a.nrows, a.b, L);
+    const int c = p.c;
     const int64_t row = p.d.x;
     T acc[R * VW];
 #pragma unroll
@@ -186,14 +208,14 @@ __global__ void __launch_bounds__(kThreads) kron_rows_kernel(const KronArgs<T> a
     constexpr int SS = MODE == KRON_CORI ? 1 : S;
     const Scatter<T, N, SS> sc(p.sp);
     constexpr int K = Scatter<T, N, SS>::kKeep;
-    const int cnt = p.on ? sc.cnt : 0;
+    const int cnt = p.n ? sc.cnt : 0;
     // a lane's own values of a block: whole vectors, or single ones when the
     // row's sums are scattered over its lane groups
     auto own = [&](const T* base, int64_t l, T (&o)[K]) {
         if constexpr (SS == 1) {
 #pragma unroll
             for (int k = 0; k < R; ++k) {
-                const Vec<T, VW> t = p.on ? ld<T, VW>(base + (R * row + k) * l + c) : zero<T, VW>();
+                const Vec<T, VW> t = ld<PAIR, T, VW>(base + (R * row + k) * l + c, p.n);
 #pragma unroll
                 for (int i = 0; i < VW; ++i) o[k * VW + i] = t.v[i];
             }
@@ -207,13 +229,13 @@ __global__ void __launch_bounds__(kThreads) kron_rows_kernel(const KronArgs<T> a
     };
     auto put = [&](T* base, int64_t l, const T (&o)[K]) {
         if constexpr (SS == 1) {
-            if (p.on && (S == 1 || p.sp == 0))
+            if (S == 1 || p.sp == 0)
 #pragma unroll
                 for (int k = 0; k < R; ++k) {
                     Vec<T, VW> t;
 #pragma unroll
                     for (int i = 0; i < VW; ++i) t.v[i] = o[k * VW + i];
-                    st<T, VW>(base + (R * row + k) * l + c, t);
+                    st<PAIR, T, VW>(base + (R * row + k) * l + c, t, p.n);
                 }
         } else {
 #pragma unroll
@@ -240,7 +262,7 @@ __global__ void __launch_bounds__(kThreads) kron_rows_kernel(const KronArgs<T> a
             in[u] = j[u] >= 0;
             vc[u] = v[u];
 #pragma unroll
-            for (int k = 0; k < R; ++k) x[u][k] = in[u] ? ld<T, VW>(X + j[u] * RL + k * a.ldx) : zero<T, VW>();
+            for (int k = 0; k < R; ++k) x[u][k] = in[u] ? ld<PAIR, T, VW>(X + j[u] * RL + k * a.ldx, p.n) : zero<T, VW>();
         }
         e += U * S;
 #pragma unroll
@@ -259,12 +281,12 @@ __global__ void __launch_bounds__(kThreads) kron_rows_kernel(const KronArgs<T> a
             }
     }
     if constexpr (SS == S) {
-        sc.sum(acc, p.sp, 1 << tl_shift);
+        sc.sum(acc, p.sp, L);
     } else {
 #pragma unroll
         for (int i = 0; i < N; ++i)
 #pragma unroll
-            for (int m = 1; m < S; m *= 2) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], m << tl_shift);
+            for (int m = 1; m < S; m *= 2) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], m * L);
     }
     T o[K];
     if (MODE == KRON_PLAIN) {
@@ -311,12 +333,12 @@ __global__ void __launch_bounds__(kThreads) kron_rows_kernel(const KronArgs<T> a
 }
 
 // ----------------------------------------------------------------- 3x3 BSR (+ E S)
-template <typename T, int VW, int S, int U>
-__global__ void __launch_bounds__(kThreads) bsr33_rows_kernel(const Bsr33Args<T> a, int tl_shift) {
-    const Place p = place<VW, S>(a.desc, a.nrows, a.b, tl_shift);
-    const int c = p.on ? p.c : 0;
+template <typename T, int VW, bool PAIR, int S, int U>
+__global__ void __launch_bounds__(kThreads) bsr33_rows_kernel(const Bsr33Args<T> a, int L) {
+    const Place p = place<VW, S>(a.desc, a.nrows, a.b, L);
+    const int c = p.c;
     const int64_t row = p.d.x;
-    const int f0 = a.e_rowptr && p.on ? __ldg(a.e_rowptr + row) : 0, f1 = a.e_rowptr && p.on ? __ldg(a.e_rowptr + row + 1) : 0;
+    const int f0 = a.e_rowptr && p.n ? __ldg(a.e_rowptr + row) : 0, f1 = a.e_rowptr && p.n ? __ldg(a.e_rowptr + row + 1) : 0;
     constexpr int N = 3 * VW;
     T acc[N];
 #pragma unroll
@@ -336,7 +358,7 @@ __global__ void __launch_bounds__(kThreads) bsr33_rows_kernel(const Bsr33Args<T>
             in[u] = j[u] >= 0;
 #pragma unroll
             for (int k = 0; k < 3; ++k)
-                x[u][k] = in[u] ? ld<T, VW>(X + (3 * (int64_t)j[u] + k) * a.ldx) : zero<T, VW>();
+                x[u][k] = in[u] ? ld<PAIR, T, VW>(X + (3 * (int64_t)j[u] + k) * a.ldx, p.n) : zero<T, VW>();
 #pragma unroll
             for (int t = 0; t < 9; ++t) kv[u][t] = in[u] ? __ldg(a.val + 9 * (int64_t)(e + u * S) + t) : T(0);
         }
@@ -357,7 +379,7 @@ __global__ void __launch_bounds__(kThreads) bsr33_rows_kernel(const Bsr33Args<T>
     }
 #pragma unroll 2
     for (int f = f0 + p.sp; f < f1; f += S) {
-        const Vec<T, VW> sv = ld<T, VW>(a.S + (int64_t)__ldg(a.e_col + f) * a.lds + c);
+        const Vec<T, VW> sv = ld<PAIR, T, VW>(a.S + (int64_t)__ldg(a.e_col + f) * a.lds + c, p.n);
 #pragma unroll
         for (int m = 0; m < 3; ++m) {
             const T ev = __ldg(a.e_val + 3 * (int64_t)f + m);
@@ -367,8 +389,8 @@ __global__ void __launch_bounds__(kThreads) bsr33_rows_kernel(const Bsr33Args<T>
     }
     const Scatter<T, N, S> sc(p.sp);
     constexpr int K = Scatter<T, N, S>::kKeep;
-    sc.sum(acc, p.sp, 1 << tl_shift);
-    if (!p.on) return;
+    sc.sum(acc, p.sp, L);
+    if (!p.n) return;
     const T d = a.X1 ? __ldg(a.dinv + row) * a.inv_theta : T(0);
     if constexpr (S == 1) {
 #pragma unroll
@@ -376,11 +398,11 @@ __global__ void __launch_bounds__(kThreads) bsr33_rows_kernel(const Bsr33Args<T>
             Vec<T, VW> t;
 #pragma unroll
             for (int i = 0; i < VW; ++i) t.v[i] = acc[m * VW + i];
-            st<T, VW>(a.W + (3 * row + m) * a.ldw + c, t);
+            st<PAIR, T, VW>(a.W + (3 * row + m) * a.ldw + c, t, p.n);
             if (a.X1) {
 #pragma unroll
                 for (int i = 0; i < VW; ++i) t.v[i] *= d;
-                st<T, VW>(a.X1 + (3 * row + m) * a.ldx1 + c, t);
+                st<PAIR, T, VW>(a.X1 + (3 * row + m) * a.ldx1 + c, t, p.n);
             }
         }
     } else {
@@ -395,10 +417,10 @@ __global__ void __launch_bounds__(kThreads) bsr33_rows_kernel(const Bsr33Args<T>
 }
 
 // ----------------------------------------------------------------- 1x3 BSR
-template <typename T, int VW, int S, int U>
-__global__ void __launch_bounds__(kThreads) bsr13_rows_kernel(const Bsr13Args<T> a, int tl_shift) {
-    const Place p = place<VW, S>(a.desc, a.nrows, a.b, tl_shift);
-    const int c = p.on ? p.c : 0;
+template <typename T, int VW, bool PAIR, int S, int U>
+__global__ void __launch_bounds__(kThreads) bsr13_rows_kernel(const Bsr13Args<T> a, int L) {
+    const Place p = place<VW, S>(a.desc, a.nrows, a.b, L);
+    const int c = p.c;
     const int64_t row = p.d.x;
     T acc[VW];
 #pragma unroll
@@ -428,7 +450,7 @@ __global__ void __launch_bounds__(kThreads) bsr13_rows_kernel(const Bsr13Args<T>
         for (int u = 0; u < U; ++u)
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                x[u][k] = in[u] ? ld<T, VW>(X + (3 * (int64_t)j[u] + k) * a.ldx) : zero<T, VW>();
+                x[u][k] = in[u] ? ld<PAIR, T, VW>(X + (3 * (int64_t)j[u] + k) * a.ldx, p.n) : zero<T, VW>();
                 vc[u][k] = v[u][k];
             }
         e += U * S;
@@ -444,12 +466,12 @@ __global__ void __launch_bounds__(kThreads) bsr13_rows_kernel(const Bsr13Args<T>
     }
     const Scatter<T, VW, S> sc(p.sp);
     constexpr int K = Scatter<T, VW, S>::kKeep;
-    sc.sum(acc, p.sp, 1 << tl_shift);
-    if (!p.on) return;
+    sc.sum(acc, p.sp, L);
+    if (!p.n) return;
     const T d = a.S1 ? __ldg(a.dinv + row) * a.inv_theta : T(0);
 #pragma unroll
     for (int i = 0; i < K; ++i) {
-        if (i >= sc.cnt) break;
+        if (i >= min(sc.cnt, S == 1 ? p.n : VW)) break;
         a.Q[row * a.ldq + c + sc.base + i] = acc[i];
         if (a.S1) a.S1[row * a.lds1 + c + sc.base + i] = d * acc[i];
     }
@@ -458,36 +480,54 @@ __global__ void __launch_bounds__(kThreads) bsr13_rows_kernel(const Bsr13Args<T>
 // ----------------------------------------------------------------- launches
 namespace {
 
+int sm_count() {
+    static std::atomic<int> n{0};
+    int v = n.load(std::memory_order_relaxed);
+    if (v == 0) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1)
+            v = 148;
+        n.store(v, std::memory_order_relaxed);
+    }
+    return v;
+}
+
 struct Shape {
-    int tl_shift, splits;
+    int vw, L, splits;
     dim3 grid;
 };
 
-// tl lanes (a power of two, at most 32) cover the columns, chunks of 32 VW
-// columns go to the grid's y; the splits double while the rows leave the chip
-// below 16 warps per SM (a double filter at 17,977 rows and 8 columns: 16.6 /
-// 15.1 / 11.7 / 12.1 ms with 4 / 8 / 16 / 32 warps).
-Shape shape(int nrows, int b, int vw) {
-    static std::atomic<int> sm_count{0};
-    int sms = sm_count.load(std::memory_order_relaxed);
-    if (sms == 0) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-            sms = 148;
-        sm_count.store(sms, std::memory_order_relaxed);
-    }
-    const int lanes = (b + vw - 1) / vw;
+// Columns per lane and lanes per row. While the rows leave the chip below 16
+// warps per SM the splits double (a double filter at 17,977 rows and 8 columns:
+// 16.6 / 15.1 / 11.7 / 12.1 ms with 4 / 8 / 16 / 32 warps); L is then a power
+// of two and the lanes hold pairs where the operands allow. Unsplit, the FP64
+// pipe bounds, and the columns per lane (1 .. 4) are those that leave fewest
+// lanes of a warp idle: 24 columns as 5 rows of 6 lanes, not 2 of 12.
+template <typename T>
+Shape shape(int nrows, int b, bool pair) {
     Shape h;
-    h.tl_shift = 0;
-    while (h.tl_shift < 5 && (1 << h.tl_shift) < lanes) ++h.tl_shift;
-    const int ny = (lanes + (1 << h.tl_shift) - 1) >> h.tl_shift;
+    h.vw = pair ? 2 : 1;
+    int lanes = (b + h.vw - 1) / h.vw, shift = 0;
+    while (shift < 5 && (1 << shift) < lanes) ++shift;
+    h.L = 1 << shift;
+    int ny = (lanes + h.L - 1) >> shift;
     h.splits = 1;
-    while (h.splits < 8 && (h.splits << h.tl_shift) < 32 &&
-           ((((int64_t)nrows * ny * h.splits) << h.tl_shift) >> 5) < 16 * (int64_t)sms)
+    while (h.splits < 8 && h.splits * h.L < 32 && (int64_t)nrows * ny * h.splits * h.L / 32 < 16 * (int64_t)sm_count())
         h.splits *= 2;
-    const int64_t threads = ((int64_t)nrows * h.splits) << h.tl_shift;
-    h.grid = dim3((unsigned)((threads + kThreads - 1) / kThreads), (unsigned)ny);
+    if (h.splits == 1 && sizeof(T) == 8) {
+        double best = 0;
+        for (int vw : {2, 4, 1, 3}) {
+            const int n = (b + vw - 1) / vw, y = (n + 31) / 32, L = (n + y - 1) / y;
+            const double use = (double)(32 / L) * b / vw / (32.0 * y);
+            if (use > best + 0.01) {
+                best = use;
+                h.vw = vw, h.L = L, ny = y;
+            }
+        }
+    }
+    const int64_t per = 32 / (h.L * h.splits) * (kThreads / 32);
+    h.grid = dim3((unsigned)((nrows + per - 1) / per), (unsigned)ny);
     return h;
 }
 
@@ -507,19 +547,7 @@ int launch(void (*k)(A...), const Shape& h, cudaStream_t s, A... args) {
     return NM_OK;
 }
 
-template <typename T, int R, int MODE, int VW>
-int kron_rows_go(const KronArgs<T>& a, cudaStream_t s) {
-    const Shape h = shape(a.nrows, a.b, VW);
-    constexpr int U = 4;
-    switch (h.splits) {
-        case 1: return launch(kron_rows_kernel<T, R, MODE, VW, 1, U>, h, s, a, h.tl_shift);
-        case 2: return launch(kron_rows_kernel<T, R, MODE, VW, 2, U>, h, s, a, h.tl_shift);
-        case 4: return launch(kron_rows_kernel<T, R, MODE, VW, 4, U>, h, s, a, h.tl_shift);
-        default: return launch(kron_rows_kernel<T, R, MODE, VW, 8, U>, h, s, a, h.tl_shift);
-    }
-}
-
-// two columns per lane need even widths and strides and aligned operands
+// two-value accesses need even widths and strides and aligned operands
 template <typename T>
 bool pairs(int b, std::initializer_list<int64_t> lds, std::initializer_list<const void*> ptrs) {
     if (b % 2) return false;
@@ -530,40 +558,56 @@ bool pairs(int b, std::initializer_list<int64_t> lds, std::initializer_list<cons
     return (p & (2 * sizeof(T) - 1)) == 0;
 }
 
+// One kernel per columns per lane, splits and kind of access.
+#define NM_ROWS(K)                                                                       \
+    if (h.splits == 1) {                                                                 \
+        switch (h.vw) {                                                                  \
+            case 1: return launch(K(1, false, 1), h, s, a, h.L);                         \
+            case 2: return pair ? launch(K(2, true, 1), h, s, a, h.L) : launch(K(2, false, 1), h, s, a, h.L); \
+            case 3: return launch(K(3, false, 1), h, s, a, h.L);                         \
+            default: return pair ? launch(K(4, true, 1), h, s, a, h.L) : launch(K(4, false, 1), h, s, a, h.L); \
+        }                                                                                \
+    }                                                                                    \
+    switch (h.splits) {                                                                  \
+        case 2: return pair ? launch(K(2, true, 2), h, s, a, h.L) : launch(K(1, false, 2), h, s, a, h.L); \
+        case 4: return pair ? launch(K(2, true, 4), h, s, a, h.L) : launch(K(1, false, 4), h, s, a, h.L); \
+        default: return pair ? launch(K(2, true, 8), h, s, a, h.L) : launch(K(1, false, 8), h, s, a, h.L); \
+    }
+
 template <typename T, int R, int MODE>
 int kron_rows_mode(const KronArgs<T>& a, cudaStream_t s) {
     if (a.nrows == 0) return NM_OK;
-    bool two;
+    bool pair;
     if (MODE == KRON_PLAIN || MODE == KRON_CORI)
-        two = pairs<T>(a.b, {a.ldx, a.ldy}, {a.X, a.Y});
+        pair = pairs<T>(a.b, {a.ldx, a.ldy}, {a.X, a.Y});
     else if (MODE == KRON_CHEB)
-        two = pairs<T>(a.b, {a.ldx, a.ldw, a.ldp, a.ldn}, {a.X, a.W, a.Xp, a.Xn});
+        pair = pairs<T>(a.b, {a.ldx, a.ldw, a.ldp, a.ldn}, {a.X, a.W, a.Xp, a.Xn});
     else
-        two = pairs<T>(a.b, {a.ldx, a.ldw, a.ldp, a.ldtk, a.ldtp, a.ldtn, a.ldz}, {a.X, a.W, a.Xp, a.Tk, a.Tp, a.Tn, a.Z});
-    return two ? kron_rows_go<T, R, MODE, 2>(a, s) : kron_rows_go<T, R, MODE, 1>(a, s);
+        pair = pairs<T>(a.b, {a.ldx, a.ldw, a.ldp, a.ldtk, a.ldtp, a.ldtn, a.ldz}, {a.X, a.W, a.Xp, a.Tk, a.Tp, a.Tn, a.Z});
+    const Shape h = shape<T>(a.nrows, a.b, pair);
+#define NM_K(VW, PAIR, S) kron_rows_kernel<T, R, MODE, VW, PAIR, S, (VW > 2 && R == 3 ? 2 : 4)>
+    NM_ROWS(NM_K)
+#undef NM_K
 }
 
-template <typename T, int VW>
-int bsr33_rows_go(const Bsr33Args<T>& a, cudaStream_t s) {
-    const Shape h = shape(a.nrows, a.b, VW);
-    switch (h.splits) {
-        case 1: return launch(bsr33_rows_kernel<T, VW, 1, 2>, h, s, a, h.tl_shift);
-        case 2: return launch(bsr33_rows_kernel<T, VW, 2, 2>, h, s, a, h.tl_shift);
-        case 4: return launch(bsr33_rows_kernel<T, VW, 4, 2>, h, s, a, h.tl_shift);
-        default: return launch(bsr33_rows_kernel<T, VW, 8, 2>, h, s, a, h.tl_shift);
-    }
+template <typename T>
+int bsr33_rows(const Bsr33Args<T>& a, cudaStream_t s) {
+    const bool pair = pairs<T>(a.b, {a.ldx, a.ldw, a.lds, a.ldx1}, {a.X, a.W, a.S, a.X1});
+    const Shape h = shape<T>(a.nrows, a.b, pair);
+#define NM_K(VW, PAIR, S) bsr33_rows_kernel<T, VW, PAIR, S, 2>
+    NM_ROWS(NM_K)
+#undef NM_K
 }
 
-template <typename T, int VW>
-int bsr13_rows_go(const Bsr13Args<T>& a, cudaStream_t s) {
-    const Shape h = shape(a.nrows, a.b, VW);
-    switch (h.splits) {
-        case 1: return launch(bsr13_rows_kernel<T, VW, 1, 4>, h, s, a, h.tl_shift);
-        case 2: return launch(bsr13_rows_kernel<T, VW, 2, 4>, h, s, a, h.tl_shift);
-        case 4: return launch(bsr13_rows_kernel<T, VW, 4, 4>, h, s, a, h.tl_shift);
-        default: return launch(bsr13_rows_kernel<T, VW, 8, 4>, h, s, a, h.tl_shift);
-    }
+template <typename T>
+int bsr13_rows(const Bsr13Args<T>& a, cudaStream_t s) {
+    const bool pair = pairs<T>(a.b, {a.ldx, a.ldq, a.lds1}, {a.X, a.Q, a.S1});
+    const Shape h = shape<T>(a.nrows, a.b, pair);
+#define NM_K(VW, PAIR, S) bsr13_rows_kernel<T, VW, PAIR, S, (VW > 2 ? 2 : 4)>
+    NM_ROWS(NM_K)
+#undef NM_K
 }
+#undef NM_ROWS
 
 }  // namespace
 
@@ -590,16 +634,14 @@ template <typename T>
 int launch_bsr33(const Bsr33Args<T>& a, cudaStream_t s) {
     if (a.b < 1 || a.b > 64) return fail(NM_EINVAL, "block width must be in 1..64");
     if (a.nrows == 0) return NM_OK;
-    return pairs<T>(a.b, {a.ldx, a.ldw, a.lds, a.ldx1}, {a.X, a.W, a.S, a.X1}) ? bsr33_rows_go<T, 2>(a, s)
-                                                                             : bsr33_rows_go<T, 1>(a, s);
+    return bsr33_rows<T>(a, s);
 }
 
 template <typename T>
 int launch_bsr13(const Bsr13Args<T>& a, cudaStream_t s) {
     if (a.b < 1 || a.b > 64) return fail(NM_EINVAL, "block width must be in 1..64");
     if (a.nrows == 0) return NM_OK;
-    return pairs<T>(a.b, {a.ldx, a.ldq, a.lds1}, {a.X, a.Q, a.S1}) ? bsr13_rows_go<T, 2>(a, s)
-                                                                  : bsr13_rows_go<T, 1>(a, s);
+    return bsr13_rows<T>(a, s);
 }
 
 // Row descriptors: rows of each window of 64 in order of decreasing length.
