@@ -30,6 +30,8 @@
 
 #include "kernels.h"
 #include "nm_internal.h"
+#include "df_convert.cuh"
+#include "df_pair.cuh"
 
 namespace nm {
 
@@ -103,75 +105,132 @@ __global__ void csr_spmm_kernel(int64_t nrows, const int64_t* __restrict__ rowpt
 
 constexpr int kTile = 128;   // targets per CTA and sources per shared-memory stage
 
-// 1/sqrt(r2) to double accuracy: the float estimate refined by one Newton
-// step for f(y) = 1/y^2 - r2, y <- y (3 - r2 y^2) / 2, which squares its
-// relative error (rsqrtf's ~1e-7 becomes ~2e-14). Four FP64 operations
-// instead of a full double-precision reciprocal square root.
-__device__ __forceinline__ double inv_dist(double r2) {
-    const double y = (double)rsqrtf((float)r2);
-    return y * fma(-0.5 * r2, y * y, 1.5);
+constexpr int kStage = 64;   // sources per shared-memory stage
+constexpr int kRun = 16;     // ... and per double-float sum
+
+// Largest exponent field of each column of Q (np x b), by atomicMax into the
+// zeroed cexp: the charges are scaled to [-2, 2) column by column, so that
+// their float pairs neither overflow nor underflow whatever the block's scale.
+__global__ void column_exp_kernel(int64_t np, int b, const double* __restrict__ Q, int* cexp) {
+    __shared__ int m[64];
+    if (threadIdx.x < 64) m[threadIdx.x] = 0;
+    __syncthreads();
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < np * b; t += (int64_t)gridDim.x * blockDim.x)
+        atomicMax(&m[t % b], (__double2hiint(Q[t]) >> 20) & 0x7FF);
+    __syncthreads();
+    if (threadIdx.x < b) atomicMax(cexp + threadIdx.x, m[threadIdx.x]);
 }
 
+// 2^(1023 - e) and 2^(e - 1023) of a column's exponent field (1 for zero, for
+// non-finite and for extreme columns).
+__device__ __forceinline__ double down_scale(int e) { return e < 1 || e > 2045 ? 1.0 : __hiloint2double((2046 - e) << 20, 0); }
+__device__ __forceinline__ double up_scale(int e) { return e < 1 || e > 2045 ? 1.0 : __hiloint2double(e << 20, 0); }
+
 // Phi[i, c] = G sum_{j != i} Q[j, c] / |r_i - r_j| + G inv_R[i] Q[i, c].
-// One thread per target and group of NC columns (blockIdx.y): one 1/r per
-// pair serves NC products, so the FP64 pipe spends ~10 of its 10 + NC
-// operations per pair on the distance. The sources pass through shared
-// memory kTile at a time. With split > 1 (small point sets, to fill the
+// One thread per target and group of NC columns (blockIdx.y). Distances and
+// products run in double-float on the float pipe (df_pair.cuh): about 60
+// operations for 1/r and 12 per column, against 9 + NC FP64 operations of 64
+// times their cost. kStage sources at a time pass through shared memory, their
+// charges as float pairs; every kRun sources the double-float sums are added
+// to running sums of three floats in shared memory (a run's own rounding, 2^-46
+// of its sum, averages out over the runs; the same additions in FP64 held its
+// pipe for 9 of 32 ms). With split > 1 (small point sets, to fill the
 // machine) CTA z sums the sources of its range [z chunk, (z + 1) chunk) into
 // part[z] and nbody_reduce_kernel adds the ranges in order.
+// Bound by the float pipe: 36,160 points, 32 columns, 444 operations a pair
+// take 15.5 ms at its peak; measured 25 ms, 98.4 ms with FP64 sums and a
+// Newton-refined 1/r (2e-14 relative).
 template <int NC>
-__global__ void __launch_bounds__(kTile) nbody_kernel(int64_t np, const double* __restrict__ pts,
+__global__ void __launch_bounds__(kTile, 3) nbody_kernel(int64_t np, const float* __restrict__ pts, double scale,
                                                      const double* __restrict__ inv_R, double G,
-                                                     const double* __restrict__ Q, int b, double* Phi,
-                                                     int64_t chunk, double* part) {
-    __shared__ double sx[kTile], sy[kTile], sz[kTile];
-    __shared__ __align__(16) double sq[kTile][NC];
+                                                     const double* __restrict__ Q, int b, const int* __restrict__ cexp,
+                                                     double* Phi, int64_t chunk, double* part) {
+    extern __shared__ __align__(16) float nb_smem[];
+    // running sums as three floats, [NC][kTile] each; volatile: loaded, added to
+    // and stored one at a time, not held in registers together
+    volatile float* const s0 = nb_smem + threadIdx.x;
+    volatile float* const s1 = s0 + NC * kTile;
+    volatile float* const s2 = s1 + NC * kTile;
+    float* const sp = nb_smem + 3 * NC * kTile;                                   // [kStage][12]
+    float2* const sq = reinterpret_cast<float2*>(sp + kStage * 12);               // [kStage][NC]
     const int c0 = blockIdx.y * NC;
     const int nc = b - c0 < NC ? b - c0 : NC;
     const int64_t i = blockIdx.x * (int64_t)kTile + threadIdx.x;
     const int64_t jb = blockIdx.z * chunk;
     const int64_t je = jb + chunk < np ? jb + chunk : np;
-    double xi = 0, yi = 0, zi = 0;
-    if (i < np) {
-        xi = pts[3 * i];
-        yi = pts[3 * i + 1];
-        zi = pts[3 * i + 2];
-    }
-    double acc[NC];
+    float xi[kLimbs];
 #pragma unroll
-    for (int c = 0; c < NC; ++c) acc[c] = 0.0;
-    for (int64_t j0 = jb; j0 < je; j0 += kTile) {
-        const int64_t j = j0 + threadIdx.x;
-        const bool in = j < je;
-        sx[threadIdx.x] = in ? pts[3 * j] : 0.0;
-        sy[threadIdx.x] = in ? pts[3 * j + 1] : 0.0;
-        sz[threadIdx.x] = in ? pts[3 * j + 2] : 0.0;
+    for (int d = 0; d < kLimbs; ++d) xi[d] = i < np ? pts[i * kLimbs + d] : 4.f;
 #pragma unroll
-        for (int c = 0; c < NC; ++c) sq[threadIdx.x][c] = (in && c < nc) ? Q[j * b + c0 + c] : 0.0;
+    for (int c = 0; c < NC; ++c) s0[c * kTile] = s1[c * kTile] = s2[c * kTile] = 0.f;
+    for (int64_t j0 = jb; j0 < je; j0 += kStage) {
+        const int cnt = je - j0 < kStage ? (int)(je - j0) : kStage;
+        for (int t = threadIdx.x; t < kStage * kLimbs; t += kTile) {
+            const int k = t / kLimbs, d = t - k * kLimbs;
+            sp[k * 12 + d] = k < cnt ? pts[(j0 + k) * kLimbs + d] : -4.f;
+        }
+        for (int t = threadIdx.x; t < kStage * NC; t += kTile) {
+            const int k = t / NC, c = t - k * NC;
+            float h = 0.f, l = 0.f;
+            if (k < cnt && c < nc) split_pair(Q[(j0 + k) * b + c0 + c] * down_scale(__ldg(cexp + c0 + c)), h, l);
+            sq[t] = make_float2(h, l);
+        }
         __syncthreads();
-        const int cnt = je - j0 < kTile ? (int)(je - j0) : kTile;
         const int64_t self = i - j0;   // the target's own slot in this stage, if any
-        for (int k = 0; k < cnt; ++k) {
-            const double dx = sx[k] - xi, dy = sy[k] - yi, dz = sz[k] - zi;
-            const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-            const double w = (k == self) ? 0.0 : inv_dist(r2);
+        for (int k0 = 0; k0 < cnt; k0 += kRun) {
+            const int k1 = min(k0 + kRun, cnt);
+            float ah[NC], al[NC];
 #pragma unroll
-            for (int c = 0; c < NC; ++c) acc[c] = fma(sq[k][c], w, acc[c]);
+            for (int c = 0; c < NC; ++c) ah[c] = al[c] = 0.f;
+#pragma unroll 1
+            for (int k = k0; k < k1; ++k) {
+                const float4* sv = reinterpret_cast<const float4*>(sp + k * 12);
+                const float4 u = sv[0], v = sv[1];
+                const float w8 = sp[k * 12 + 8];
+                float h[3], l[3], y, e, q, ql;
+                limb_diff(u.x, u.w, v.z, xi[0], xi[3], xi[6], h[0], l[0]);
+                limb_diff(u.y, v.x, v.w, xi[1], xi[4], xi[7], h[1], l[1]);
+                limb_diff(u.z, v.y, w8, xi[2], xi[5], xi[8], h[2], l[2]);
+                inv_dist_df(h, l, y, e, q, ql);
+                float wl = __fmul_rn(y, __fmul_rn(e, __fmaf_rn(0.375f, e, 0.5f)));
+                if (k == self) y = wl = 0.f;
+                const float4* qv = reinterpret_cast<const float4*>(sq + k * NC);
+#pragma unroll
+                for (int c = 0; c < NC; c += 2) {
+                    const float4 t = qv[c / 2];
+                    df_add(ah[c], al[c], y, wl, t.x, t.y);
+                    df_add(ah[c + 1], al[c + 1], y, wl, t.z, t.w);
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                float a, t, e1, e2, e3;
+                two_sum(s0[c * kTile], ah[c], a, e1);
+                s0[c * kTile] = a;
+                two_sum(s1[c * kTile], e1, t, e2);
+                two_sum(t, al[c], a, e3);
+                s1[c * kTile] = a;
+                s2[c * kTile] = __fadd_rn(s2[c * kTile], __fadd_rn(e2, e3));
+            }
         }
         __syncthreads();
     }
     if (i >= np) return;
+    auto sum = [&](int c) {
+        return scale * up_scale(__ldg(cexp + c0 + c)) *
+               ((double)s0[c * kTile] + ((double)s1[c * kTile] + (double)s2[c * kTile]));
+    };
     if (part) {
         double* o = part + ((int64_t)blockIdx.z * np + i) * b + c0;
 #pragma unroll
         for (int c = 0; c < NC; ++c)
-            if (c < nc) o[c] = acc[c];
+            if (c < nc) o[c] = sum(c);
         return;
     }
     const double d = inv_R[i];
 #pragma unroll
     for (int c = 0; c < NC; ++c)
-        if (c < nc) Phi[i * b + c0 + c] = G * fma(d, Q[i * b + c0 + c], acc[c]);
+        if (c < nc) Phi[i * b + c0 + c] = G * fma(d, Q[i * b + c0 + c], sum(c));
 }
 
 // Phi = G (sum over the source ranges of part + inv_R Q), ranges in order.
@@ -207,19 +266,27 @@ int nbody_split(int64_t np, int b) {
 }
 
 template <int NC>
-void launch_nbody(int64_t np, const double* pts, const double* inv_R, double G, const double* Q, int b, double* Phi,
-                  double* part, cudaStream_t s) {
+int launch_nbody(int64_t np, const float* pts, double scale, const double* inv_R, double G, const double* Q, int b,
+                 int* cexp, double* Phi, double* part, cudaStream_t s) {
     const int split = nbody_split(np, b);
     const int64_t tiles = (np + kTile - 1) / kTile;
     const int64_t chunk = ((tiles + split - 1) / split) * kTile;
     dim3 grid((unsigned)tiles, (unsigned)((b + NC - 1) / NC), (unsigned)split);
-    nbody_kernel<NC><<<grid, kTile, 0, s>>>(np, pts, inv_R, G, Q, b, Phi, chunk, split > 1 ? part : nullptr);
+    constexpr size_t smem = (size_t)NC * kTile * 12 + kStage * 12 * 4 + (size_t)kStage * NC * 8;
+    NM_CUDA(cudaFuncSetAttribute(nbody_kernel<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    NM_CUDA(cudaMemsetAsync(cexp, 0, 64 * sizeof(int), s));
+    column_exp_kernel<<<(unsigned)std::min<int64_t>((np * b + 4095) / 4096, 1024), 256, 0, s>>>(np, b, Q, cexp);
+    count_launch();
+    nbody_kernel<NC><<<grid, kTile, smem, s>>>(np, pts, scale, inv_R, G, Q, b, cexp, Phi, chunk, split > 1 ? part : nullptr);
     if (split > 1) {
         count_launch();
         const int64_t total = np * b;
         const int blocks = (int)std::min<int64_t>((total + 255) / 256, 4096);
         nbody_reduce_kernel<<<blocks, 256, 0, s>>>(np, b, split, part, inv_R, G, Q, Phi);
     }
+    count_launch();
+    NM_CUDA(cudaGetLastError());
+    return NM_OK;
 }
 
 struct Entry {
@@ -430,6 +497,16 @@ int build_self_gravity(nm_problem* P, const double* xyz, const int32_t* tet, con
     NM_TRY(SG.invR.alloc(invR.size() * sizeof(double)));
     NM_CUDA(cudaMemcpy(SG.pts.p, pts.data(), pts.size() * sizeof(double), cudaMemcpyHostToDevice));
     NM_CUDA(cudaMemcpy(SG.invR.p, invR.data(), invR.size() * sizeof(double), cudaMemcpyHostToDevice));
+    // the points in limbs, scaled by a power of two to [-1, 1]
+    double far = 0;
+    for (double v : pts) far = std::max(far, std::fabs(v));
+    SG.inv_scale = far > 0 ? std::exp2(-std::ceil(std::log2(far))) : 1.0;
+    NM_TRY(SG.cexp.alloc(64 * sizeof(int)));
+    NM_TRY(SG.limbs.alloc(np * kLimbs * sizeof(float)));
+    split_points_kernel<<<1024, 256, 0, P->ctx->stream>>>(np, 3, SG.pts.as<double>(), SG.inv_scale, SG.limbs.as<float>());
+    count_launch();
+    NM_CUDA(cudaGetLastError());
+    NM_CUDA(cudaStreamSynchronize(P->ctx->stream));
     std::vector<Entry> tr(ent.size());
     for (size_t k = 0; k < ent.size(); ++k) tr[k] = {ent[k].col, (int32_t)ent[k].row, ent[k].val};
     NM_TRY(upload_csr(ent, np, SG.c_rp, SG.c_col, SG.c_val));
@@ -460,16 +537,15 @@ int apply_selfgrav(nm_problem* P, const double* X, int64_t ldx, double* W, int64
     count_launch();
     NM_CUDA(cudaGetLastError());
     // the narrowest column group that holds the block (wider blocks: groups of 32)
-    const double *pts = SG.pts.as<double>(), *invR = SG.invR.as<double>(), *q = SG.q.as<double>();
+    const double *invR = SG.invR.as<double>(), *q = SG.q.as<double>();
+    const float* pts = SG.limbs.as<float>();
     double *phi = SG.phi.as<double>(), *part = SG.part.as<double>();
     if (nbody_cols(b) == 8)
-        launch_nbody<8>(SG.np, pts, invR, SG.G, q, b, phi, part, s);
+        NM_TRY(launch_nbody<8>(SG.np, pts, SG.inv_scale, invR, SG.G, q, b, SG.cexp.as<int>(), phi, part, s));
     else if (nbody_cols(b) == 16)
-        launch_nbody<16>(SG.np, pts, invR, SG.G, q, b, phi, part, s);
+        NM_TRY(launch_nbody<16>(SG.np, pts, SG.inv_scale, invR, SG.G, q, b, SG.cexp.as<int>(), phi, part, s));
     else
-        launch_nbody<32>(SG.np, pts, invR, SG.G, q, b, phi, part, s);
-    count_launch();
-    NM_CUDA(cudaGetLastError());
+        NM_TRY(launch_nbody<32>(SG.np, pts, SG.inv_scale, invR, SG.G, q, b, SG.cexp.as<int>(), phi, part, s));
     csr_spmm_kernel<<<(unsigned)((n + per - 1) / per), 256, 0, s>>>(
         n, SG.t_rp.as<int64_t>(), SG.t_col.as<int>(), SG.t_val.as<double>(), SG.phi.as<double>(), b, W, ldw, b, -1.0,
         1.0);

@@ -170,3 +170,21 @@ def test_slice_of_the_full_planet_pencil(nm, sg_planet):
     assert np.allclose(res.lam, ref, rtol=1e-8, atol=1e-10 * lam[-1])
     assert res.resid.max() <= 1e-6
     res.free()
+
+
+@pytest.mark.parametrize("b,scale", [(3, 1.0), (16, 1e-60), (33, 1e60)])
+def test_potential_sum_is_linear_in_scale(sg_planet, b, scale):
+    """The direct sum runs in float pairs on columns scaled to unit size: a
+    block of any magnitude gives the same product times its scale (FP64 form,
+    1e-11 as above; column 1 is zero, column 2 nine orders smaller)."""
+    mesh, model, S, T, P = sg_planet
+    Xc = np.random.default_rng(b).standard_normal((S.n, b))
+    Xc[:, 1] = 0.0
+    Xc[:, 2] *= 1e-9
+    Y = torch.empty((S.n, b), dtype=torch.float64, device=DEV)
+    P.apply_K(torch.tensor(to_internal(P, Xc) * scale, device=DEV), Y, k_P=80)
+    got = to_canonical(P, Y.cpu().numpy()) / scale
+    op = filtlan.Operator(S, k_M=10, k_P=80)
+    ref = op.K(Xc) - T @ Xc
+    for c in range(b):
+        assert np.abs(got[:, c] - ref[:, c]).max() <= 1e-11 * np.abs(ref[:, c]).max()
