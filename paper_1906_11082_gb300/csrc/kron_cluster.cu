@@ -32,6 +32,7 @@
 
 #include "kernels.h"
 #include "nm_internal.h"
+#include "dependent.cuh"
 
 namespace nm {
 
@@ -58,10 +59,17 @@ __device__ __forceinline__ void fma2(unsigned long long& d, unsigned long long a
 struct F4 {
     unsigned long long lo, hi;
 };
+// NC: by the read-only path
+template <bool NC>
 __device__ __forceinline__ F4 ldg4(const float* p) {
-    F4 r;
-    asm("ld.global.nc.v2.b64 {%0, %1}, [%2];" : "=l"(r.lo), "=l"(r.hi) : "l"(p));
-    return r;
+    if constexpr (NC) {
+        F4 r;
+        asm("ld.global.nc.v2.b64 {%0, %1}, [%2];" : "=l"(r.lo), "=l"(r.hi) : "l"(p));
+        return r;
+    } else {
+        const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(p);
+        return {t.x, t.y};
+    }
 }
 __device__ __forceinline__ float4 f4(const F4& v) {
     const float2 a = unpack2(v.lo), b = unpack2(v.hi);
@@ -72,7 +80,7 @@ __device__ __forceinline__ float4 f4(const F4& v) {
 
 // L: 16-byte columns of a column group (grid y); DENSE: the gathered block is
 // exactly one group wide. Lane (cluster cw of the warp, split sp, column q).
-template <int R, int L, int MODE, int S, int U, bool DENSE, int MINB>
+template <int R, int L, int MODE, int S, int U, bool DENSE, bool DEP, int MINB>
 __global__ void __launch_bounds__(kThreads, MINB) kron_cluster_kernel(const KronArgs<float> a) {
     constexpr int LC = S * L;                 // lanes of a cluster
     constexpr int CW = 32 / LC;               // clusters of a warp
@@ -94,6 +102,9 @@ __global__ void __launch_bounds__(kThreads, MINB) kron_cluster_kernel(const Kron
     int c[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) c[u] = __ldg(a.cl.col + min(e + sp + u * S, e1 - 1));
+    // DEP: started while the previous step drains. What is loaded above is
+    // matrix data; the blocks are read after this wait, and by plain loads.
+    if constexpr (DEP) dep_sync();
     for (int first = (blockIdx.x * (kThreads / 32) + warp) * CW; first <= last; first += stride) {
         const bool on = cw < CW && cl <= last && q < nq;
         const int cn = min(cl + stride, last);
@@ -128,7 +139,7 @@ __global__ void __launch_bounds__(kThreads, MINB) kron_cluster_kernel(const Kron
             for (int u = 0; u < U; ++u) {
                 const float* p = X + c[u] * (R * ld);
 #pragma unroll
-                for (int k = 0; k < R; ++k) x[u][k] = ldg4(p + k * ld);
+                for (int k = 0; k < R; ++k) x[u][k] = ldg4<!DEP>(p + k * ld);
             }
 #pragma unroll
             for (int u = 0; u < U; ++u) {
@@ -228,7 +239,8 @@ __global__ void __launch_bounds__(kThreads, MINB) kron_cluster_kernel(const Kron
             const float dd = pd[i] * a.inv_theta;
 #pragma unroll
             for (int k = 0; k < R; ++k) {
-                const float4 xk = __ldg(reinterpret_cast<const float4*>(X + ((int64_t)R * row[i] + k) * ld));
+                const float4* px = reinterpret_cast<const float4*>(X + ((int64_t)R * row[i] + k) * ld);
+                const float4 xk = DEP ? *px : __ldg(px);
                 const float4 xp = pp[i][k], w = pw[i][k];
                 float4 sm = sum[i][k];
                 // a non-finite record times a zero value of another row: the row's own entries decide
@@ -237,7 +249,7 @@ __global__ void __launch_bounds__(kThreads, MINB) kron_cluster_kernel(const Kron
                     sm = make_float4(0.f, 0.f, 0.f, 0.f);
                     for (int j = __ldg(a.rowptr + row[i]); j < __ldg(a.rowptr + row[i] + 1); ++j) {
                         const float vj = __ldg(a.val + j);
-                        const float4 xj = __ldg(reinterpret_cast<const float4*>(X + ((int64_t)R * __ldg(a.col + j) + k) * ld));
+                        const float4 xj = f4(ldg4<!DEP>(X + ((int64_t)R * __ldg(a.col + j) + k) * ld));
                         sm.x = fmaf(vj, xj.x, sm.x);
                         sm.y = fmaf(vj, xj.y, sm.y);
                         sm.z = fmaf(vj, xj.z, sm.z);
@@ -280,10 +292,18 @@ template <int R, int L, int MODE, int S, int U, int MINB>
 static int cluster_go(const KronArgs<float>& a, int ng, cudaStream_t s) {
     const int64_t per = 32 / (S * L) * (kThreads / 32);
     const unsigned grid = (unsigned)std::min<int64_t>((a.cl.n + per - 1) / per, (int64_t)a.cl.sms * MINB);
-    if (a.ldx == 4 * L && ng == 1)
-        kron_cluster_kernel<R, L, MODE, S, U, true, MINB><<<dim3(grid, 1), kThreads, 0, s>>>(a);
-    else
-        kron_cluster_kernel<R, L, MODE, S, U, false, MINB><<<dim3(grid, ng), kThreads, 0, s>>>(a);
+    if (a.ldx == 4 * L && ng == 1) {
+        // Steps of less than about 20 warps per SM start while their
+        // predecessor drains (803 clusters, 24 columns: a filter of 1,200
+        // steps 10.9 -> 8.0 ms; 16.6k clusters, 16 columns 16.6 -> 15.6 ms);
+        // above, the early CTAs and the plain loads cost more than the gap
+        // (96k clusters, 32 columns 100.9 -> 104.0 ms).
+        if ((int64_t)a.cl.n * L < 640 * (int64_t)a.cl.sms)
+            return launch_dependent(kron_cluster_kernel<R, L, MODE, S, U, true, true, MINB>, dim3(grid), kThreads, s, a);
+        kron_cluster_kernel<R, L, MODE, S, U, true, false, MINB><<<grid, kThreads, 0, s>>>(a);
+    } else {
+        kron_cluster_kernel<R, L, MODE, S, U, false, false, MINB><<<dim3(grid, ng), kThreads, 0, s>>>(a);
+    }
     count_launch();
     NM_CUDA(cudaGetLastError());
     return NM_OK;

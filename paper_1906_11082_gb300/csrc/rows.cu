@@ -32,6 +32,7 @@
 
 #include "kernels.h"
 #include "nm_internal.h"
+#include "dependent.cuh"
 
 namespace nm {
 
@@ -96,15 +97,6 @@ __device__ __forceinline__ Vec<T, VW> zero() {
 #pragma unroll
     for (int i = 0; i < VW; ++i) r.v[i] = T(0);
     return r;
-}
-
-// Wait for the predecessor's results, then let the successor start: only two
-// kernels of a chain are ever in flight together. What is loaded before this
-// point is matrix data no kernel of a chain writes; blocks are read after it,
-// by plain (not read-only path) loads.
-__device__ __forceinline__ void dep_sync() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Sums N values over the S lane groups (tl lanes each) of a row. Every step
@@ -531,22 +523,6 @@ Shape shape(int nrows, int b, bool pair) {
     return h;
 }
 
-template <typename... A>
-int launch(void (*k)(A...), const Shape& h, cudaStream_t s, A... args) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = h.grid;
-    cfg.blockDim = dim3(kThreads);
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    NM_CUDA(cudaLaunchKernelEx(&cfg, k, args...));
-    count_launch();
-    return NM_OK;
-}
-
 // two-value accesses need even widths and strides and aligned operands
 template <typename T>
 bool pairs(int b, std::initializer_list<int64_t> lds, std::initializer_list<const void*> ptrs) {
@@ -562,16 +538,16 @@ bool pairs(int b, std::initializer_list<int64_t> lds, std::initializer_list<cons
 #define NM_ROWS(K)                                                                       \
     if (h.splits == 1) {                                                                 \
         switch (h.vw) {                                                                  \
-            case 1: return launch(K(1, false, 1), h, s, a, h.L);                         \
-            case 2: return pair ? launch(K(2, true, 1), h, s, a, h.L) : launch(K(2, false, 1), h, s, a, h.L); \
-            case 3: return launch(K(3, false, 1), h, s, a, h.L);                         \
-            default: return pair ? launch(K(4, true, 1), h, s, a, h.L) : launch(K(4, false, 1), h, s, a, h.L); \
+            case 1: return launch_dependent(K(1, false, 1), h.grid, kThreads, s, a, h.L);                         \
+            case 2: return pair ? launch_dependent(K(2, true, 1), h.grid, kThreads, s, a, h.L) : launch_dependent(K(2, false, 1), h.grid, kThreads, s, a, h.L); \
+            case 3: return launch_dependent(K(3, false, 1), h.grid, kThreads, s, a, h.L);                         \
+            default: return pair ? launch_dependent(K(4, true, 1), h.grid, kThreads, s, a, h.L) : launch_dependent(K(4, false, 1), h.grid, kThreads, s, a, h.L); \
         }                                                                                \
     }                                                                                    \
     switch (h.splits) {                                                                  \
-        case 2: return pair ? launch(K(2, true, 2), h, s, a, h.L) : launch(K(1, false, 2), h, s, a, h.L); \
-        case 4: return pair ? launch(K(2, true, 4), h, s, a, h.L) : launch(K(1, false, 4), h, s, a, h.L); \
-        default: return pair ? launch(K(2, true, 8), h, s, a, h.L) : launch(K(1, false, 8), h, s, a, h.L); \
+        case 2: return pair ? launch_dependent(K(2, true, 2), h.grid, kThreads, s, a, h.L) : launch_dependent(K(1, false, 2), h.grid, kThreads, s, a, h.L); \
+        case 4: return pair ? launch_dependent(K(2, true, 4), h.grid, kThreads, s, a, h.L) : launch_dependent(K(1, false, 4), h.grid, kThreads, s, a, h.L); \
+        default: return pair ? launch_dependent(K(2, true, 8), h.grid, kThreads, s, a, h.L) : launch_dependent(K(1, false, 8), h.grid, kThreads, s, a, h.L); \
     }
 
 template <typename T, int R, int MODE>
