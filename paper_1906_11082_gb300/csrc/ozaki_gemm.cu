@@ -411,10 +411,11 @@ int ozaki_gemm_tn(nm_ctx* ctx, cudaStream_t s, int64_t I, int64_t J, int64_t K, 
     const int64_t chunks = std::max<int64_t>((K + kChunk - 1) / kChunk, 1);
     // One CTA per SM in all. A CTA's terms are summed in parts of at most 32
     // chunks, since one running FP64 sum over all of them rounds once per
-    // chunk.
+    // chunk; longer parts where the workspace would pass 64 MB.
     const int64_t ctas = std::max<int64_t>(1, std::min<int64_t>(chunks, sm_count() / (ti * tj)));
     const int64_t per_cta = (chunks + ctas - 1) / ctas;
-    const int64_t ppc = (per_cta + 31) / 32, cpp = (per_cta + ppc - 1) / ppc;
+    const int64_t room = std::max<int64_t>(1, (64ll << 20) / (8 * I * J * ctas));
+    const int64_t ppc = std::min<int64_t>((per_cta + 31) / 32, room), cpp = (per_cta + ppc - 1) / ppc;
     const int64_t nz = (chunks + ppc * cpp - 1) / (ppc * cpp);
     const int64_t parts = std::max<int64_t>(1, (chunks + cpp - 1) / cpp);
     const size_t need = (size_t)parts * I * J * sizeof(double);
