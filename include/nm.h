@@ -201,15 +201,14 @@ int nm_problem_export(const nm_problem* prob, int which, int64_t* nrows, int64_t
  * own contiguous range of rows in a single wave (CTA size = the value, L1
  * preferred over shared memory); 0 (default) turns it off; it takes
  * precedence over the other schedules. key "vec": 1 (default) runs the float semi-iteration SpMMs
- * of blocks exactly 32 wide with ld = 32 with 16-byte vectorised gathers
- * (each row split over four groups of eight lanes), 0 with one 4-byte
- * gather per lane and component; key "vec_threads" (32 default, 64, 128,
- * 256, 512, 1024; one row per warp) sets their CTA size for the
- * 3-component mass rows, "vec_threads_p" (128 default) for the
- * 1-component pressure rows: larger CTAs put more consecutive rows on one
- * SM's L1, smaller ones free their slot sooner when a CTA's rows differ in
- * length. key "df_threads" (32 default, 64, 128, 256): CTA size of the
- * NM_MIXED form's lane-group double-float SpMMs (b = 32). key "overlap":
+ * on clusters of four rows that share neighbours, with 16-byte gathers (the
+ * clusters are built on the host on first use), 0 row by row; the products
+ * without a semi-iteration and the "sched" order of 32-column float blocks
+ * split each row over four groups of eight lanes instead: key "vec_threads"
+ * (32 default, 64, 128, 256, 512, 1024; one row per warp) sets the CTA size
+ * of those kernels for 3-component rows, "vec_threads_p" (128 default) for
+ * 1-component ones. key "df_threads" (32 default, 64, 128, 256): accepted
+ * for programs that set it; the double-float SpMMs' CTA size is fixed. key "overlap":
  * 1 runs the mixed-form K_eff's fluid pressure chain (E_G^T X, the refined
  * A_p solve) on a high-priority second stream of the problem while the A_G
  * product runs on the caller's stream, then adds E_G S; 0 (default) runs
@@ -235,7 +234,7 @@ int nm_problem_export(const nm_problem* prob, int which, int64_t* nrows, int64_t
  * warps compute the previous tiles; the tiles (at most 32 rows and 160
  * distinct neighbours) are built on the host on first use. Its waits are
  * bounded: a wait that runs out makes the next nm_lanczos_step return
- * NM_ETIMEOUT. 0 (default) uses the lane-group kernel. NM_EINVAL for an
+ * NM_ETIMEOUT. 0 (default) uses the row clusters. NM_EINVAL for an
  * unknown key or value. */
 int nm_set_option(nm_problem* prob, const char* key, int64_t value);
 
