@@ -75,17 +75,17 @@ SERVING_MESHES = [(0.25, 58954.0), (0.15, 45045.0), (0.1, 85700.0)]
 SERVING_SLICES = [(4.0, 5.5), (4.5, 6.0), (3.5, 5.0)]
 
 # ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch of the
-# float mass-step kernel (kron_v4_kernel<3, 1, 32>) on this workload (same
+# float mass-step kernel (kron_cluster_kernel<3, 8>) on this workload (same
 # matrices, b = 32; mean of two launches), captured with
 #   ncu --kernel-name-base demangled --metrics gpu__time_duration.sum,\
 #       dram__bytes_read.sum,dram__bytes_write.sum --clock-control none \
-#       -k 'regex:kron_v4_kernel<\(int\)3' -s 4 -c 2 --csv \
+#       -k 'regex:kron_cluster_kernel<.int.3, .int.8' -s 4 -c 2 --csv \
 #       python bench.py --profile-case filter
-# and the SHA-256 of kernels.cu when it was taken: once the kernel source
+# and the SHA-256 of kron_cluster.cu when it was taken: once the kernel source
 # changes the figure no longer describes it and the bench reports traffic
 # null.
-TRAFFIC_CAPTURE = {"kernel": "kron_v4_kernel<3, 1, 32>", "bytes": 543_591_808 + 121_877_248,
-                   "kernels_cu_sha256": "2d86c3f12eacd75a3d36d4645078875c2e42d76cb1c6fc99cd683f8038ef0bf0"}
+TRAFFIC_CAPTURE = {"kernel": "kron_cluster_kernel<3, 8>", "bytes": 570_886_784 + 124_145_664,
+                   "kernel_sha256": "25da5ade7a2f24bf627739e814e1db7ded87261c26b555f17135624c22b99292"}
 
 # FP64 peak of GB300 (NVIDIA's published B300 figure, 1.25 TFLOP/s; equal to
 # 152 SMs x ~2.05 GHz x 2 FP64 FMA per SM per clock x 2 flop).
@@ -236,7 +236,7 @@ def peaks():
 
 
 def kernels_sha256():
-    with open(os.path.join(ROOT, "paper_1906_11082_gb300", "csrc", "kernels.cu"), "rb") as f:
+    with open(os.path.join(ROOT, "paper_1906_11082_gb300", "csrc", "kron_cluster.cu"), "rb") as f:
         return hashlib.sha256(f.read()).hexdigest()
 
 
@@ -641,16 +641,16 @@ def run_ours(args):
     gbs = mbytes / avg_launch_s / 1e9 if dl else None
     tfl = mflops / avg_launch_s / 1e12 if dl else None
     traffic = None
-    if (s == 4 and args.h == H_MESH and TRAFFIC_CAPTURE["kernels_cu_sha256"] == kernels_sha256()):
+    if (s == 4 and args.h == H_MESH and TRAFFIC_CAPTURE["kernel_sha256"] == kernels_sha256()):
         traffic = TRAFFIC_CAPTURE["bytes"]
     if args.prec == "f64" and tfl is not None and tfl / FP64_PEAK_TFLOPS > gbs / peak_hbm:
         roof = {"bound": "alu", "achieved": tfl, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                "frac": tfl / FP64_PEAK_TFLOPS, "traffic": None, "kernel": "kron_warp_kernel<double, 3, 1, 1>",
+                "frac": tfl / FP64_PEAK_TFLOPS, "traffic": None, "kernel": "kron_rows_kernel<double, 3>",
                 "peak_source": "GB300 FP64 nominal (152 SM x 2 FMA/clk x 2.05 GHz)"}
     else:
         roof = {"bound": "hbm", "achieved": gbs, "peak": peak_hbm, "unit": "GB/s",
                 "frac": (gbs / peak_hbm) if gbs else None, "traffic": traffic,
-                "kernel": "kron_warp_kernel<double, 3, 1, 1>" if s == 8 else TRAFFIC_CAPTURE["kernel"],
+                "kernel": "kron_rows_kernel<double, 3>" if s == 8 else TRAFFIC_CAPTURE["kernel"],
                 "peak_source": f"{peak_src} copy bandwidth"}
     roof["bytes_per_launch"] = mbytes
     roof["flops_per_launch"] = mflops
