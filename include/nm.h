@@ -431,11 +431,11 @@ int nm_ritz(nm_problem* prob, nm_ritz_mode mode, const double* V, int64_t ldv, i
  * The dense algebra of the block Lanczos and the Ritz projections (Sec. 6.2:
  * the Gram-Schmidt coefficients V^T M W and updates W - V C; Rayleigh-Ritz
  * V^T K V, V^T M V and X = V S; Sec. 7: X^T R X) in FP64 accuracy on the
- * tensor cores: each operand is cut into eight exact 7-bit pieces per
+ * tensor cores: each operand is cut into seven exact base-256 digits per
  * chunk of 64 contraction terms (scaled to the largest entry of its row or
- * column in the chunk), the 36 leading piece products run as bf16 tensor-
+ * column in the chunk), the 34 leading digit products run as fp16 tensor-
  * core products with exact float accumulation, and the chunk sums are
- * added in FP64. The error is of the order of 2^-53 times the sum over the
+ * put together in integers and added in FP64. The error is of the order of 2^-53 times the sum over the
  * contraction of the products of each row's and column's largest entries.
  * Deterministic (fixed split and summation order). All pointers device.
  * nm_gemm_tn: C (I x J, column-major, ld ldc) = alpha X^T Y + beta C with

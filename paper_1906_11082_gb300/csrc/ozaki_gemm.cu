@@ -28,15 +28,16 @@
 // TN splits the long contraction over CTAs into a fixed number of parts
 // summed in order by a second kernel, so every result is deterministic.
 //
-// What bounds it: the FP64 pipe and the splitting before, the tensor cores'
-// mma.sync rate now. With eight 7-bit pieces combined in FP64 per diagonal
+// What bounds it: the FP64 pipe and the splitting before; now the latency of
+// cutting operands between products with two warps per scheduler (234 to 254
+// registers), not yet the mma.sync rate. With eight 7-bit pieces combined in FP64 per diagonal
 // (about 12 FP64 operations per output and chunk) and the splitting redone by
 // every warp for every 16 output columns, V^T W at n = 1.15M, 576 x 32 took
 // 22.0 ms and V C 23.5 ms. Now a warp holds 16 rows by 32 columns: an X entry
 // is cut once (about 20 integer instructions, packed fp16 conversion), a Y
 // entry once per CTA into shared memory in fragment order, raw chunks arrive
-// by cp.async one chunk ahead: 6.6 ms and 6.2 ms, the mma.sync pipe busy 40%
-// of the time (its limit 2.5 ms; 10.9 GB for both would take 1.6 ms).
+// by cp.async one chunk ahead: 6.8 ms and 6.0 ms, the mma.sync pipe busy 39 to
+// 40% of the time (its limit 2.5 ms each; 10.9 GB for both would take 1.6 ms).
 #include <algorithm>
 #include <cstdint>
 
