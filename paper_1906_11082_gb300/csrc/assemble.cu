@@ -1086,11 +1086,16 @@ __global__ void lo_part_kernel(int64_t n, const double* v, const float* hi, floa
         lo[t] = __double2float_rn(v[t] - (double)hi[t]);
 }
 
+// Matrix data made on first use is complete before the call goes on: kernels
+// launched while their predecessor drains (dependent.cuh) load it before they
+// wait for that predecessor, and a later call may come on another stream.
 static int to_f32(DevCSR& A, cudaStream_t s) {
     if (A.nnz == 0 || A.val32.p) return NM_OK;
     const int64_t cnt = A.nnz * A.rb * A.cb;
     NM_TRY(A.val32.alloc(cnt * sizeof(float)));
-    return launch_d2f(cnt, A.val.as<double>(), A.val32.as<float>(), s);
+    NM_TRY(launch_d2f(cnt, A.val.as<double>(), A.val32.as<float>(), s));
+    NM_CUDA(cudaStreamSynchronize(s));
+    return NM_OK;
 }
 
 // What the float semi-iterations of the mixed form need: float values and
@@ -1114,10 +1119,12 @@ int ensure_df(nm_problem* P, cudaStream_t s) {
             A->nnz, A->val.as<double>(), A->val32.as<float>(), A->vlo32.as<float>());
         count_launch();
         NM_CUDA(cudaGetLastError());
+        NM_CUDA(cudaStreamSynchronize(s));
     }
     if (P->AG.nnz > 0 && !P->AG.rec.p) {
         NM_TRY(P->AG.rec.alloc(P->AG.nnz * 5 * sizeof(float4)));
         NM_TRY(launch_df_records(P->AG.nnz, P->AG.val.as<double>(), P->AG.rec.as<float4>(), s));
+        NM_CUDA(cudaStreamSynchronize(s));
     }
     return NM_OK;
 }

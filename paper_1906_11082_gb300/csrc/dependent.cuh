@@ -10,8 +10,10 @@ namespace nm {
 
 // Wait for the predecessor's results, then let the successor start: only two
 // kernels of a chain are ever in flight together. What is loaded before this
-// point is matrix data no kernel of a chain writes; blocks are read after it,
-// by plain (not read-only path) loads.
+// point is matrix data, which no kernel in flight writes: the host waits for the
+// kernels that make it, at assembly and on first use (to_f32, ensure_df,
+// build_clusters). Blocks are read after it, by plain (not read-only path)
+// loads.
 __device__ __forceinline__ void dep_sync() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
