@@ -81,6 +81,13 @@ int DevBuf::alloc(size_t nbytes) {
     return NM_OK;
 }
 
+int copy_in(void* dst, const void* src, size_t bytes, cudaStream_t s) {
+    if (bytes == 0) return NM_OK;
+    NM_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s));
+    NM_CUDA(cudaStreamSynchronize(s));
+    return NM_OK;
+}
+
 void DevBuf::release() {
     if (p) cudaFree(p);
     p = nullptr;

@@ -572,23 +572,22 @@ static void scatter_positions(const std::vector<int32_t>& rowptr, const std::vec
 }
 
 template <class T>
-static int upload(DevBuf& buf, const std::vector<T>& h) {
+static int upload(DevBuf& buf, const std::vector<T>& h, cudaStream_t s) {
     NM_TRY(buf.alloc(std::max<size_t>(h.size(), 1) * sizeof(T)));
-    if (!h.empty()) NM_CUDA(cudaMemcpy(buf.p, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice));
-    return NM_OK;
+    return copy_in(buf.p, h.data(), h.size() * sizeof(T), s);
 }
 
 static int upload_pattern(DevCSR& A, int64_t nrows, int64_t ncols, int rb, int cb,
-                          std::vector<int32_t>&& rp, std::vector<int32_t>&& col) {
+                          std::vector<int32_t>&& rp, std::vector<int32_t>&& col, cudaStream_t s) {
     A.nrows = nrows;
     A.ncols = ncols;
     A.nnz = rp.empty() ? 0 : rp.back();
     A.rb = rb;
     A.cb = cb;
-    NM_TRY(upload(A.rowptr, rp));
-    NM_TRY(upload(A.col, col));
+    NM_TRY(upload(A.rowptr, rp, s));
+    NM_TRY(upload(A.col, col, s));
     NM_TRY(A.val.alloc(std::max<int64_t>(A.nnz, 1) * rb * cb * sizeof(double)));
-    NM_CUDA(cudaMemset(A.val.p, 0, std::max<int64_t>(A.nnz, 1) * rb * cb * sizeof(double)));
+    NM_CUDA(cudaMemsetAsync(A.val.p, 0, std::max<int64_t>(A.nnz, 1) * rb * cb * sizeof(double), s));
     A.h_rowptr = std::move(rp);
     A.h_col = std::move(col);
     return NM_OK;
@@ -596,7 +595,7 @@ static int upload_pattern(DevCSR& A, int64_t nrows, int64_t ncols, int rb, int c
 
 // Row tiles of a scalar square pattern (see DevCSR): the distinct columns of
 // each tile of `rows` consecutive rows and every entry's local position.
-static int build_tiles(DevCSR& A, int rows) {
+static int build_tiles(DevCSR& A, int rows, cudaStream_t s) {
     const int64_t n = A.nrows;
     A.tile_rows = rows;
     A.ntiles = (n + rows - 1) / rows;
@@ -618,9 +617,9 @@ static int build_tiles(DevCSR& A, int rows) {
         uptr[t + 1] = (int32_t)ucol.size();
     }
     A.tile_umax = umax;
-    NM_TRY(upload(A.tile_uptr, uptr));
-    NM_TRY(upload(A.tile_ucol, ucol));
-    NM_TRY(upload(A.lcol, lcol));
+    NM_TRY(upload(A.tile_uptr, uptr, s));
+    NM_TRY(upload(A.tile_ucol, ucol, s));
+    NM_TRY(upload(A.lcol, lcol, s));
     return NM_OK;
 }
 
@@ -637,8 +636,8 @@ int set_tile_rows(nm_problem* P, int64_t rows) {
         return NM_OK;
     }
     if (rows < 4 || rows > 64 || (rows & (rows - 1))) return fail(NM_EINVAL, "tile_rows must be 0 or 4..64, a power of two");
-    NM_TRY(build_tiles(P->Mr, (int)rows));
-    if (P->info.Np > 0) NM_TRY(build_tiles(P->Pn, (int)rows));
+    NM_TRY(build_tiles(P->Mr, (int)rows, P->ctx->stream));
+    if (P->info.Np > 0) NM_TRY(build_tiles(P->Pn, (int)rows, P->ctx->stream));
     if ((size_t)P->Mr.tile_umax * 3 * 32 * sizeof(float) > 200 * 1024)
         return fail(NM_EINVAL, "tile_rows too large: staged operand exceeds shared memory");
     return NM_OK;
@@ -691,7 +690,9 @@ int assemble(nm_ctx* ctx, const nm_mesh* mesh, const nm_model* mdl, nm_problem* 
     if (nfluid > 0 && (!mdl->N2 && gravity)) return fail(NM_EINVAL, "N2 is required with fluid tets and gravity");
     RefMats R;
     NM_TRY(build_reference(R));
-    NM_CUDA(cudaMemcpyToSymbol(cRef, &R, sizeof(RefMats)));
+    cudaStream_t s = ctx->stream;
+    NM_CUDA(cudaMemcpyToSymbolAsync(cRef, &R, sizeof(RefMats), 0, cudaMemcpyHostToDevice, s));
+    NM_CUDA(cudaStreamSynchronize(s));
 
     // ---- P2 nodes: vertices then edges in lexicographic (min, max) order
     std::vector<int64_t> ekey(6 * nt);
@@ -856,9 +857,9 @@ int assemble(nm_ctx* ctx, const nm_mesh* mesh, const nm_model* mdl, nm_problem* 
     ElemGroup gf{nfs, 6, 6, fs_us.data(), fs_us.data()};
     if (nfs) scatter_positions(rp, cl, gf, posFU);
     std::vector<int32_t> rp2(rp), cl2(cl);
-    NM_TRY(upload_pattern(P->AG, Nu, Nu, 3, 3, std::move(rp), std::move(cl)));
-    NM_TRY(upload_pattern(P->Mr, Nu, Nu, 1, 1, std::move(rp2), std::move(cl2)));
-    NM_TRY(build_row_desc(P->Mr));   // A_G has the same pattern
+    NM_TRY(upload_pattern(P->AG, Nu, Nu, 3, 3, std::move(rp), std::move(cl), s));
+    NM_TRY(upload_pattern(P->Mr, Nu, Nu, 1, 1, std::move(rp2), std::move(cl2), s));
+    NM_TRY(build_row_desc(P->Mr, s));   // A_G has the same pattern
 
     std::vector<int64_t> ftets;
     std::vector<int32_t> ftu, ftp;   // fluid tets: u-nodes and p-nodes
@@ -881,36 +882,51 @@ int assemble(nm_ctx* ctx, const nm_mesh* mesh, const nm_model* mdl, nm_problem* 
         std::vector<int32_t> a, b;
         NM_TRY(build_pattern(Np, {gpp}, a, b));
         scatter_positions(a, b, gpp, posP);
-        NM_TRY(upload_pattern(P->Pn, Np, Np, 1, 1, std::move(a), std::move(b)));
-        NM_TRY(build_row_desc(P->Pn));
+        NM_TRY(upload_pattern(P->Pn, Np, Np, 1, 1, std::move(a), std::move(b), s));
+        NM_TRY(build_row_desc(P->Pn, s));
         std::vector<int32_t> c, d;
         NM_TRY(build_pattern(Nu, {gup, gfup}, c, d));
         scatter_positions(c, d, gup, posE);
         if (nfs) scatter_positions(c, d, gfup, posFE);
-        NM_TRY(upload_pattern(P->EG, Nu, Np, 3, 1, std::move(c), std::move(d)));
+        NM_TRY(upload_pattern(P->EG, Nu, Np, 3, 1, std::move(c), std::move(d), s));
         std::vector<int32_t> e, f;
         NM_TRY(build_pattern(Np, {gpu, gfpu}, e, f));
         scatter_positions(e, f, gpu, posEt);
         if (nfs) scatter_positions(e, f, gfpu, posFEt);
-        NM_TRY(upload_pattern(P->EGt, Np, Nu, 1, 3, std::move(e), std::move(f)));
-        NM_TRY(build_row_desc(P->EGt));
+        NM_TRY(upload_pattern(P->EGt, Np, Nu, 1, 3, std::move(e), std::move(f), s));
+        NM_TRY(build_row_desc(P->EGt, s));
     }
 
     // ---- device inputs
-    cudaStream_t s = ctx->stream;
     DevBuf d_vx, d_tu, d_reg, d_rho, d_lam, d_mu, d_N2, d_posU;
     std::vector<double> vx(12 * nt);
     for (int64_t t = 0; t < nt; ++t)
         for (int a = 0; a < 4; ++a)
             for (int d = 0; d < 3; ++d) vx[12 * t + 3 * a + d] = xyz[3 * tet[4 * t + a] + d];
-    NM_TRY(upload(d_vx, vx));
-    NM_TRY(upload(d_tu, tu));
-    NM_TRY(upload(d_reg, std::vector<uint8_t>(mesh->region, mesh->region + nt)));
-    NM_TRY(upload(d_rho, std::vector<double>(mdl->rho, mdl->rho + nt)));
-    NM_TRY(upload(d_lam, std::vector<double>(mdl->lam, mdl->lam + nt)));
-    NM_TRY(upload(d_mu, std::vector<double>(mdl->mu, mdl->mu + nt)));
-    NM_TRY(upload(d_N2, mdl->N2 ? std::vector<double>(mdl->N2, mdl->N2 + nt) : std::vector<double>(nt, 0.0)));
-    NM_TRY(upload(d_posU, posU));
+    NM_TRY(upload(d_vx, vx, s));
+    NM_TRY(upload(d_tu, tu, s));
+    NM_TRY(upload(d_reg, std::vector<uint8_t>(mesh->region, mesh->region + nt), s));
+    NM_TRY(upload(d_rho, std::vector<double>(mdl->rho, mdl->rho + nt), s));
+    NM_TRY(upload(d_lam, std::vector<double>(mdl->lam, mdl->lam + nt), s));
+    NM_TRY(upload(d_mu, std::vector<double>(mdl->mu, mdl->mu + nt), s));
+    NM_TRY(upload(d_N2, mdl->N2 ? std::vector<double>(mdl->N2, mdl->N2 + nt) : std::vector<double>(nt, 0.0), s));
+    NM_TRY(upload(d_posU, posU, s));
+    DevBuf d_ftets, d_posP, d_posE, d_posEt, d_fn, d_fa, d_frho, d_fus, d_posFU, d_posFE, d_posFEt;
+    if (Np > 0) {
+        NM_TRY(upload(d_ftets, ftets, s));
+        NM_TRY(upload(d_posP, posP, s));
+        NM_TRY(upload(d_posE, posE, s));
+        NM_TRY(upload(d_posEt, posEt, s));
+        if (nfs > 0) {
+            NM_TRY(upload(d_fn, fs_n, s));
+            NM_TRY(upload(d_fa, fs_a, s));
+            NM_TRY(upload(d_frho, fs_rho, s));
+            NM_TRY(upload(d_fus, fs_us, s));
+            NM_TRY(upload(d_posFU, posFU, s));
+            NM_TRY(upload(d_posFE, posFE, s));
+            NM_TRY(upload(d_posFEt, posFEt, s));
+        }
+    }
 
     // ---- reference field g' at the u-nodes
     NM_TRY(P->g.alloc(3 * Nu * sizeof(double)));
@@ -920,7 +936,7 @@ int assemble(nm_ctx* ctx, const nm_mesh* mesh, const nm_model* mdl, nm_problem* 
             std::vector<double> gh(3 * Nu);
             for (int64_t i = 0; i < Nu; ++i)
                 for (int d = 0; d < 3; ++d) gh[3 * i + d] = mdl->gprime[3 * P->p2_of_internal[i] + d];
-            NM_CUDA(cudaMemcpy(P->g.p, gh.data(), gh.size() * sizeof(double), cudaMemcpyHostToDevice));
+            NM_TRY(copy_in(P->g.p, gh.data(), gh.size() * sizeof(double), s));
         } else {
             std::vector<double> ux(3 * Nu), src(4 * nt);
             for (int64_t i = 0; i < Nu; ++i)
@@ -940,8 +956,8 @@ int assemble(nm_ctx* ctx, const nm_mesh* mesh, const nm_model* mdl, nm_problem* 
                 src[4 * t + 3] = mdl->rho[t] * std::fabs(det) / 6.0;
             }
             DevBuf d_ux, d_src;
-            NM_TRY(upload(d_ux, ux));
-            NM_TRY(upload(d_src, src));
+            NM_TRY(upload(d_ux, ux, s));
+            NM_TRY(upload(d_src, src, s));
             double far = 0, mmax = 0, emin = 1e300;
             for (int d = 0; d < 3; ++d) far = std::max(far, std::max(std::fabs(lo[d]), std::fabs(hi[d])));
             for (int64_t t = 0; t < nt; ++t) {
@@ -991,12 +1007,7 @@ int assemble(nm_ctx* ctx, const nm_mesh* mesh, const nm_model* mdl, nm_problem* 
     elem_u_kernel<<<(unsigned)nt, 128, 0, s>>>(ea);
     count_launch();
         NM_CUDA(cudaGetLastError());
-    DevBuf d_ftets, d_posP, d_posE, d_posEt, d_fn, d_fa, d_frho, d_fus, d_posFU, d_posFE, d_posFEt;
     if (Np > 0) {
-        NM_TRY(upload(d_ftets, ftets));
-        NM_TRY(upload(d_posP, posP));
-        NM_TRY(upload(d_posE, posE));
-        NM_TRY(upload(d_posEt, posEt));
         FluidArgs fa{nft, d_ftets.as<int64_t>(), d_vx.as<double>(), d_tu.as<int>(), d_rho.as<double>(),
                      d_lam.as<double>(), d_mu.as<double>(), gravity ? P->g.as<double>() : nullptr,
                      d_posP.as<int>(), d_posE.as<int>(), d_posEt.as<int>(), P->Pn.val.as<double>(),
@@ -1005,13 +1016,6 @@ int assemble(nm_ctx* ctx, const nm_mesh* mesh, const nm_model* mdl, nm_problem* 
         count_launch();
         NM_CUDA(cudaGetLastError());
         if (nfs > 0) {
-            NM_TRY(upload(d_fn, fs_n));
-            NM_TRY(upload(d_fa, fs_a));
-            NM_TRY(upload(d_frho, fs_rho));
-            NM_TRY(upload(d_fus, fs_us));
-            NM_TRY(upload(d_posFU, posFU));
-            NM_TRY(upload(d_posFE, posFE));
-            NM_TRY(upload(d_posFEt, posFEt));
             FaceArgs fc{nfs, d_fn.as<double>(), d_fa.as<double>(), d_frho.as<double>(), d_fus.as<int>(),
                         gravity ? P->g.as<double>() : nullptr, d_posFU.as<int>(), d_posFE.as<int>(),
                         d_posFEt.as<int>(), P->AG.val.as<double>(), P->EG.val.as<double>(),
@@ -1032,7 +1036,7 @@ int assemble(nm_ctx* ctx, const nm_mesh* mesh, const nm_model* mdl, nm_problem* 
             dpos[i] = it - A.h_col.data();
         }
         DevBuf d_dpos;
-        NM_TRY(upload(d_dpos, dpos));
+        NM_TRY(upload(d_dpos, dpos, s));
         NM_TRY(A.dinv.alloc(std::max<int64_t>(A.nrows, 1) * sizeof(double)));
         NM_TRY(A.dinv32.alloc(std::max<int64_t>(A.nrows, 1) * sizeof(float)));
         dinv_kernel<<<(unsigned)std::min<int64_t>((A.nrows + 255) / 256 + 1, 4096), 256, 0, s>>>(

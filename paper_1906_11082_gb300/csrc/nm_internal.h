@@ -103,9 +103,14 @@ struct DevCSR {
     DevBuf tma_desc, tma_ucol, tma_lcol, tma_vals, tma_rowptr, tma_dinv, tma_ldiag, tma_err;
 };
 
+// Host to device in the order of stream s, complete on return. The contexts'
+// streams are not ordered with the legacy stream, and a plain copy from pageable
+// memory returns once the data is staged, before it has reached the device:
+// what a kernel on s reads has to be copied on s.
+int copy_in(void* dst, const void* src, size_t bytes, cudaStream_t s);
 int build_tma_tiles(DevCSR& A, cudaStream_t s);
 int build_clusters(DevCSR& A, cudaStream_t s);
-int build_row_desc(DevCSR& A);
+int build_row_desc(DevCSR& A, cudaStream_t s);
 
 struct Workspace {
     DevBuf buf;      // filter recurrence scratch

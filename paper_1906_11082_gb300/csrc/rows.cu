@@ -621,7 +621,7 @@ int launch_bsr13(const Bsr13Args<T>& a, cudaStream_t s) {
 }
 
 // Row descriptors: rows of each window of 64 in order of decreasing length.
-int build_row_desc(DevCSR& A) {
+int build_row_desc(DevCSR& A, cudaStream_t s) {
     const int64_t N = A.nrows;
     std::vector<int4> d(std::max<int64_t>(N, 1));
     const int32_t* rp = A.h_rowptr.data();
@@ -632,8 +632,7 @@ int build_row_desc(DevCSR& A) {
         std::stable_sort(d.begin() + r0, d.begin() + r1, [](const int4& x, const int4& y) { return x.z - x.y > y.z - y.y; });
     }
     NM_TRY(A.desc.alloc(d.size() * sizeof(int4)));
-    NM_CUDA(cudaMemcpy(A.desc.p, d.data(), d.size() * sizeof(int4), cudaMemcpyHostToDevice));
-    return NM_OK;
+    return copy_in(A.desc.p, d.data(), d.size() * sizeof(int4), s);
 }
 
 template int launch_kron_rows<double>(int, int, const KronArgs<double>&, cudaStream_t);

@@ -295,7 +295,7 @@ struct Entry {
     double val;
 };
 
-int upload_csr(std::vector<Entry>& ent, int64_t nrows, DevBuf& rp, DevBuf& cl, DevBuf& vl) {
+int upload_csr(std::vector<Entry>& ent, int64_t nrows, DevBuf& rp, DevBuf& cl, DevBuf& vl, cudaStream_t s) {
     std::sort(ent.begin(), ent.end(), [](const Entry& a, const Entry& b) {
         return a.row != b.row ? a.row < b.row : a.col < b.col;
     });
@@ -315,12 +315,9 @@ int upload_csr(std::vector<Entry>& ent, int64_t nrows, DevBuf& rp, DevBuf& cl, D
     NM_TRY(rp.alloc(h_rp.size() * sizeof(int64_t)));
     NM_TRY(cl.alloc(std::max<size_t>(h_c.size(), 1) * sizeof(int32_t)));
     NM_TRY(vl.alloc(std::max<size_t>(h_v.size(), 1) * sizeof(double)));
-    NM_CUDA(cudaMemcpy(rp.p, h_rp.data(), h_rp.size() * sizeof(int64_t), cudaMemcpyHostToDevice));
-    if (!h_c.empty()) {
-        NM_CUDA(cudaMemcpy(cl.p, h_c.data(), h_c.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
-        NM_CUDA(cudaMemcpy(vl.p, h_v.data(), h_v.size() * sizeof(double), cudaMemcpyHostToDevice));
-    }
-    return NM_OK;
+    NM_TRY(copy_in(rp.p, h_rp.data(), h_rp.size() * sizeof(int64_t), s));
+    NM_TRY(copy_in(cl.p, h_c.data(), h_c.size() * sizeof(int32_t), s));
+    return copy_in(vl.p, h_v.data(), h_v.size() * sizeof(double), s);
 }
 
 }  // namespace
@@ -495,22 +492,23 @@ int build_self_gravity(nm_problem* P, const double* xyz, const int32_t* tet, con
     SG.G = G;
     NM_TRY(SG.pts.alloc(pts.size() * sizeof(double)));
     NM_TRY(SG.invR.alloc(invR.size() * sizeof(double)));
-    NM_CUDA(cudaMemcpy(SG.pts.p, pts.data(), pts.size() * sizeof(double), cudaMemcpyHostToDevice));
-    NM_CUDA(cudaMemcpy(SG.invR.p, invR.data(), invR.size() * sizeof(double), cudaMemcpyHostToDevice));
+    cudaStream_t s = P->ctx->stream;
+    NM_TRY(copy_in(SG.pts.p, pts.data(), pts.size() * sizeof(double), s));
+    NM_TRY(copy_in(SG.invR.p, invR.data(), invR.size() * sizeof(double), s));
     // the points in limbs, scaled by a power of two to [-1, 1]
     double far = 0;
     for (double v : pts) far = std::max(far, std::fabs(v));
     SG.inv_scale = far > 0 ? std::exp2(-std::ceil(std::log2(far))) : 1.0;
     NM_TRY(SG.cexp.alloc(64 * sizeof(int)));
     NM_TRY(SG.limbs.alloc(np * kLimbs * sizeof(float)));
-    split_points_kernel<<<1024, 256, 0, P->ctx->stream>>>(np, 3, SG.pts.as<double>(), SG.inv_scale, SG.limbs.as<float>());
+    split_points_kernel<<<1024, 256, 0, s>>>(np, 3, SG.pts.as<double>(), SG.inv_scale, SG.limbs.as<float>());
     count_launch();
     NM_CUDA(cudaGetLastError());
-    NM_CUDA(cudaStreamSynchronize(P->ctx->stream));
+    NM_CUDA(cudaStreamSynchronize(s));
     std::vector<Entry> tr(ent.size());
     for (size_t k = 0; k < ent.size(); ++k) tr[k] = {ent[k].col, (int32_t)ent[k].row, ent[k].val};
-    NM_TRY(upload_csr(ent, np, SG.c_rp, SG.c_col, SG.c_val));
-    NM_TRY(upload_csr(tr, n, SG.t_rp, SG.t_col, SG.t_val));
+    NM_TRY(upload_csr(ent, np, SG.c_rp, SG.c_col, SG.c_val, s));
+    NM_TRY(upload_csr(tr, n, SG.t_rp, SG.t_col, SG.t_val, s));
     NM_TRY(SG.q.alloc((size_t)np * 64 * sizeof(double)));
     NM_TRY(SG.phi.alloc((size_t)np * 64 * sizeof(double)));
     // partial sums of the split n-body launches, for the widest need over b

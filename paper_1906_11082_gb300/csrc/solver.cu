@@ -1384,7 +1384,7 @@ static int rayleigh_ritz(nm_problem* P, const double* V, int64_t ldv, int m, dou
             k = (int)keep.size();
             if (k > 0) {
                 NM_TRY(Skeep.alloc(hk.size() * sizeof(double)));
-                NM_CUDA(cudaMemcpy(Skeep.p, hk.data(), hk.size() * sizeof(double), cudaMemcpyHostToDevice));
+                NM_TRY(copy_in(Skeep.p, hk.data(), hk.size() * sizeof(double), s));
                 Ssel = Skeep.as<double>();
             }
         }
@@ -1487,7 +1487,7 @@ int spectrum_bounds(nm_problem* P, int steps, int k_M, uint64_t seed, double* la
     DevBuf Td, wd;
     NM_TRY(Td.alloc((size_t)m * m * sizeof(double)));
     NM_TRY(wd.alloc((size_t)m * sizeof(double)));
-    NM_CUDA(cudaMemcpy(Td.p, Tm.data(), Tm.size() * sizeof(double), cudaMemcpyHostToDevice));
+    NM_TRY(copy_in(Td.p, Tm.data(), Tm.size() * sizeof(double), s));
     NM_TRY(dense_eig(ctx, m, Td.as<double>(), nullptr, wd.as<double>()));
     std::vector<double> th(m), Sv((size_t)m * m);
     NM_CUDA(cudaMemcpy(th.data(), wd.p, m * sizeof(double), cudaMemcpyDeviceToHost));
@@ -1751,7 +1751,7 @@ int lanczos_step(nm_lanczos* L, int* active_out) {
             DevBuf Td, wd;
             NM_TRY(Td.alloc(Tm.size() * sizeof(double)));
             NM_TRY(wd.alloc(m * sizeof(double)));
-            NM_CUDA(cudaMemcpy(Td.p, Tm.data(), Tm.size() * sizeof(double), cudaMemcpyHostToDevice));
+            NM_TRY(copy_in(Td.p, Tm.data(), Tm.size() * sizeof(double), s));
             NM_TRY(dense_eig(ctx, m, Td.as<double>(), nullptr, wd.as<double>()));
             std::vector<double> th(m), Sv((size_t)m * m);
             NM_CUDA(cudaMemcpy(th.data(), wd.p, m * sizeof(double), cudaMemcpyDeviceToHost));
@@ -2002,8 +2002,8 @@ int ritz(nm_problem* P, nm_ritz_mode mode, const double* V, int64_t ldv, int m, 
         NM_TRY(Bd.alloc(B.size() * sizeof(cuDoubleComplex)));
         NM_TRY(wd.alloc(m2 * sizeof(double)));
         NM_TRY(info.alloc(sizeof(int)));
-        NM_CUDA(cudaMemcpy(Ad.p, A.data(), A.size() * sizeof(cuDoubleComplex), cudaMemcpyHostToDevice));
-        NM_CUDA(cudaMemcpy(Bd.p, B.data(), B.size() * sizeof(cuDoubleComplex), cudaMemcpyHostToDevice));
+        NM_TRY(copy_in(Ad.p, A.data(), A.size() * sizeof(cuDoubleComplex), s));
+        NM_TRY(copy_in(Bd.p, B.data(), B.size() * sizeof(cuDoubleComplex), s));
         int lwork = 0;
         NM_CUSOLVER(cusolverDnZhegvd_bufferSize(ctx->cusolver, CUSOLVER_EIG_TYPE_1, CUSOLVER_EIG_MODE_VECTOR,
                                                 CUBLAS_FILL_MODE_UPPER, m2, Ad.as<cuDoubleComplex>(), m2,
@@ -2048,8 +2048,8 @@ int ritz(nm_problem* P, nm_ritz_mode mode, const double* V, int64_t ldv, int m, 
             NM_TRY(yid.alloc(yi.size() * sizeof(double)));
             NM_TRY(Ur.alloc((size_t)n * k * sizeof(double)));
             NM_TRY(Ui.alloc((size_t)n * k * sizeof(double)));
-            NM_CUDA(cudaMemcpy(yrd.p, yr.data(), yr.size() * sizeof(double), cudaMemcpyHostToDevice));
-            NM_CUDA(cudaMemcpy(yid.p, yi.data(), yi.size() * sizeof(double), cudaMemcpyHostToDevice));
+            NM_TRY(copy_in(yrd.p, yr.data(), yr.size() * sizeof(double), s));
+            NM_TRY(copy_in(yid.p, yi.data(), yi.size() * sizeof(double), s));
             NM_TRY(gemm_VS(ctx, n, m, k, V, ldv, yrd.as<double>(), m, Ur.as<double>(), k));
             NM_TRY(gemm_VS(ctx, n, m, k, V, ldv, yid.as<double>(), m, Ui.as<double>(), k));
             // full quadratic residual ||w^2 M u - 2 i w R u - K u|| / ||w^2 M u|| (reported, not gated)
