@@ -73,11 +73,11 @@ typedef enum { NM_RITZ_PENCIL = 0, NM_RITZ_ROTATING = 1 } nm_ritz_mode;
  * fluid-solid faces (the density jump times int_E nu . u, at the face
  * barycentre); S is G / |r_i - r_j| between points and G / R_i on the
  * diagonal, 1/R_i the mean of 1/|x - r_i| over the point's own element or
- * face. Applied by a direct FP64 sum over the points (O(points^2) per
+ * face. Applied by a direct sum over the points (O(points^2) per
  * column, points ~ tets + boundary faces; its point buffers, 2 * 64
- * doubles per point, are allocated at assembly). Supported with NM_F64 and
- * NM_MIXED (the term is applied in double); NM_F32 products return
- * NM_EUNSUPPORTED. */
+ * doubles per point, are allocated at assembly): in FP64 with NM_F64, and
+ * with NM_MIXED in the arithmetic that the option "double_float" chooses for
+ * its products (nm_set_option). NM_F32 products return NM_EUNSUPPORTED. */
 #define NM_SELF_GRAVITY  4u
 
 typedef struct nm_ctx nm_ctx;
@@ -223,10 +223,11 @@ int nm_problem_export(const nm_problem* prob, int which, int64_t* nrows, int64_t
  * rebuilt on the host. key "tile_kernel": 1 or 2, the staged kernel
  * variant (256-thread rounds / 512-thread unrolled rounds). key
  * "double_float": 1 (default) runs the NM_MIXED form's double-precision
- * SpMMs (the K_eff block SpMM and the refinement residuals) as
- * double-float arithmetic on the float units (values split exactly into
- * two floats, error-free products and sums, ~2^-48 relative); 0 runs them
- * in double. key "tma": 1 runs the float mass steps of 32-column blocks
+ * SpMMs (the K_eff block SpMM and the refinement residuals) and the sums of
+ * the self-gravitation term as double-float arithmetic on the float units
+ * (values split exactly into two floats, error-free products and sums, ~2^-48
+ * relative; a pair of the self-gravitation sums ~2^-46, unbiased); 0 runs
+ * them in double. key "tma": 1 runs the float mass steps of 32-column blocks
  * (ld 32) as the shared-memory staged kernel: persistent CTAs whose
  * producer warps copy each row tile's distinct neighbour records into a
  * three-stage shared-memory ring (cp.async, with cp.async.bulk for the

@@ -166,7 +166,8 @@ void self_gravity_host(const double* xyz, const int32_t* tet, const int64_t* tet
                        std::vector<double>& pts, std::vector<double>& invR, std::vector<int64_t>& erow,
                        std::vector<int32_t>& ecol, std::vector<double>& eval);
 // W -= C^T S C X, X and W row-major n x b (b <= 64) in double.
-int apply_selfgrav(nm_problem* P, const double* X, int64_t ldx, double* W, int64_t ldw, int b, cudaStream_t s);
+int apply_selfgrav(nm_problem* P, const double* X, int64_t ldx, double* W, int64_t ldw, int b, bool df,
+                   cudaStream_t s);
 }  // namespace nm
 
 struct nm_problem {

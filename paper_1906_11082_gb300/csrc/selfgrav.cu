@@ -16,9 +16,10 @@
 // 1/R_i the mean of 1/|x - r_i| over the point's own element or face.
 //
 // Here the charges are a sparse matrix C (points x dofs, built on the host
-// at assembly), the point-to-point sum is a direct N-body kernel in FP64,
-// and apply_selfgrav subtracts C^T S C X from a K_eff product. The direct
-// sum costs O(points^2) per column; the paper applies S by FMM.
+// at assembly), the point-to-point sum is a direct N-body kernel, and
+// apply_selfgrav subtracts C^T S C X from a K_eff product: in FP64 for the
+// double form, in double-float for the mixed form's double-float products. The
+// direct sum costs O(points^2) per column; the paper applies S by FMM.
 //
 // The self distances are integrated in polar coordinates about the foot of
 // the barycentre in each face plane, in closed form (element:
@@ -103,9 +104,81 @@ __global__ void csr_spmm_kernel(int64_t nrows, const int64_t* __restrict__ rowpt
     if (lane + 32 < b) y[lane + 32] = alpha * s1 + (beta == 0.0 ? 0.0 : beta * y[lane + 32]);
 }
 
-constexpr int kTile = 128;   // targets per CTA and sources per shared-memory stage
+constexpr int kTile = 128;   // targets per CTA (and sources per shared-memory stage of the FP64 kernel)
 
-constexpr int kStage = 64;   // sources per shared-memory stage
+// 1/sqrt(r2) to double accuracy: the float estimate refined by one Newton
+// step for f(y) = 1/y^2 - r2, y <- y (3 - r2 y^2) / 2, which squares its
+// relative error (rsqrtf's ~1e-7 becomes ~2e-14). Four FP64 operations
+// instead of a full double-precision reciprocal square root.
+__device__ __forceinline__ double inv_dist(double r2) {
+    const double y = (double)rsqrtf((float)r2);
+    return y * fma(-0.5 * r2, y * y, 1.5);
+}
+
+// Phi[i, c] = G sum_{j != i} Q[j, c] / |r_i - r_j| + G inv_R[i] Q[i, c] in FP64.
+// One thread per target and group of NC columns (blockIdx.y): one 1/r per
+// pair serves NC products, so the FP64 pipe spends ~10 of its 10 + NC
+// operations per pair on the distance. The sources pass through shared
+// memory kTile at a time. With split > 1 (small point sets, to fill the
+// machine) CTA z sums the sources of its range [z chunk, (z + 1) chunk) into
+// part[z] and nbody_reduce_kernel adds the ranges in order. Bound by the FP64
+// pipe: 36,160 points, 32 columns 98 ms.
+template <int NC>
+__global__ void __launch_bounds__(kTile) nbody_kernel(int64_t np, const double* __restrict__ pts,
+                                                     const double* __restrict__ inv_R, double G,
+                                                     const double* __restrict__ Q, int b, double* Phi,
+                                                     int64_t chunk, double* part) {
+    __shared__ double sx[kTile], sy[kTile], sz[kTile];
+    __shared__ __align__(16) double sq[kTile][NC];
+    const int c0 = blockIdx.y * NC;
+    const int nc = b - c0 < NC ? b - c0 : NC;
+    const int64_t i = blockIdx.x * (int64_t)kTile + threadIdx.x;
+    const int64_t jb = blockIdx.z * chunk;
+    const int64_t je = jb + chunk < np ? jb + chunk : np;
+    double xi = 0, yi = 0, zi = 0;
+    if (i < np) {
+        xi = pts[3 * i];
+        yi = pts[3 * i + 1];
+        zi = pts[3 * i + 2];
+    }
+    double acc[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) acc[c] = 0.0;
+    for (int64_t j0 = jb; j0 < je; j0 += kTile) {
+        const int64_t j = j0 + threadIdx.x;
+        const bool in = j < je;
+        sx[threadIdx.x] = in ? pts[3 * j] : 0.0;
+        sy[threadIdx.x] = in ? pts[3 * j + 1] : 0.0;
+        sz[threadIdx.x] = in ? pts[3 * j + 2] : 0.0;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) sq[threadIdx.x][c] = (in && c < nc) ? Q[j * b + c0 + c] : 0.0;
+        __syncthreads();
+        const int cnt = je - j0 < kTile ? (int)(je - j0) : kTile;
+        const int64_t self = i - j0;   // the target's own slot in this stage, if any
+        for (int k = 0; k < cnt; ++k) {
+            const double dx = sx[k] - xi, dy = sy[k] - yi, dz = sz[k] - zi;
+            const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+            const double w = (k == self) ? 0.0 : inv_dist(r2);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) acc[c] = fma(sq[k][c], w, acc[c]);
+        }
+        __syncthreads();
+    }
+    if (i >= np) return;
+    if (part) {
+        double* o = part + ((int64_t)blockIdx.z * np + i) * b + c0;
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+            if (c < nc) o[c] = acc[c];
+        return;
+    }
+    const double d = inv_R[i];
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+        if (c < nc) Phi[i * b + c0 + c] = G * fma(d, Q[i * b + c0 + c], acc[c]);
+}
+
+constexpr int kStage = 64;   // sources per shared-memory stage of the double-float kernel
 constexpr int kRun = 16;     // ... and per double-float sum
 
 // Largest exponent field of each column of Q (np x b), by atomicMax into the
@@ -126,22 +199,21 @@ __global__ void column_exp_kernel(int64_t np, int b, const double* __restrict__ 
 __device__ __forceinline__ double down_scale(int e) { return e < 1 || e > 2045 ? 1.0 : __hiloint2double((2046 - e) << 20, 0); }
 __device__ __forceinline__ double up_scale(int e) { return e < 1 || e > 2045 ? 1.0 : __hiloint2double(e << 20, 0); }
 
-// Phi[i, c] = G sum_{j != i} Q[j, c] / |r_i - r_j| + G inv_R[i] Q[i, c].
-// One thread per target and group of NC columns (blockIdx.y). Distances and
-// products run in double-float on the float pipe (df_pair.cuh): about 60
+// The same sums in double-float on the float pipe (df_pair.cuh): about 60
 // operations for 1/r and 12 per column, against 9 + NC FP64 operations of 64
 // times their cost. kStage sources at a time pass through shared memory, their
 // charges as float pairs; every kRun sources the double-float sums are added
-// to running sums of three floats in shared memory (a run's own rounding, 2^-46
-// of its sum, averages out over the runs; the same additions in FP64 held its
-// pipe for 9 of 32 ms). With split > 1 (small point sets, to fill the
-// machine) CTA z sums the sources of its range [z chunk, (z + 1) chunk) into
-// part[z] and nbody_reduce_kernel adds the ranges in order.
+// to running sums of three floats in shared memory (the same additions in FP64
+// held its pipe for 9 of 32 ms). A pair and its additions err by about 1e-14
+// of a term, unbiased: against quad precision, 6,100 to 133,360 points, the
+// potential of random charges errs by 4e-15 to 6e-15 of its largest value
+// (root mean square), by 1.3e-15 to 2.9e-15 with nbody_kernel; that of charges
+// of one sign by 3e-16 to 1.3e-15 against 1.0e-15 to 1.2e-15, whose 1/r is
+// biased. Hence the mixed form only, whose option "double_float" chooses.
 // Bound by the float pipe: 36,160 points, 32 columns, 444 operations a pair
-// take 15.5 ms at its peak; measured 25 ms, 98.4 ms with FP64 sums and a
-// Newton-refined 1/r (2e-14 relative).
+// take 15.5 ms at its peak; measured 25 ms.
 template <int NC>
-__global__ void __launch_bounds__(kTile, 3) nbody_kernel(int64_t np, const float* __restrict__ pts, double scale,
+__global__ void __launch_bounds__(kTile, 3) nbody_df_kernel(int64_t np, const float* __restrict__ pts, double scale,
                                                      const double* __restrict__ inv_R, double G,
                                                      const double* __restrict__ Q, int b, const int* __restrict__ cexp,
                                                      double* Phi, int64_t chunk, double* part) {
@@ -266,23 +338,32 @@ int nbody_split(int64_t np, int b) {
 }
 
 template <int NC>
-int launch_nbody(int64_t np, const float* pts, double scale, const double* inv_R, double G, const double* Q, int b,
-                 int* cexp, double* Phi, double* part, cudaStream_t s) {
+int launch_nbody(SelfGravity& SG, bool df, int b, cudaStream_t s) {
+    const int64_t np = SG.np;
+    const double *invR = SG.invR.as<double>(), *Q = SG.q.as<double>();
+    double* Phi = SG.phi.as<double>();
     const int split = nbody_split(np, b);
+    double* part = split > 1 ? SG.part.as<double>() : nullptr;
     const int64_t tiles = (np + kTile - 1) / kTile;
     const int64_t chunk = ((tiles + split - 1) / split) * kTile;
     dim3 grid((unsigned)tiles, (unsigned)((b + NC - 1) / NC), (unsigned)split);
-    constexpr size_t smem = (size_t)NC * kTile * 12 + kStage * 12 * 4 + (size_t)kStage * NC * 8;
-    NM_CUDA(cudaFuncSetAttribute(nbody_kernel<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    NM_CUDA(cudaMemsetAsync(cexp, 0, 64 * sizeof(int), s));
-    column_exp_kernel<<<(unsigned)std::min<int64_t>((np * b + 4095) / 4096, 1024), 256, 0, s>>>(np, b, Q, cexp);
-    count_launch();
-    nbody_kernel<NC><<<grid, kTile, smem, s>>>(np, pts, scale, inv_R, G, Q, b, cexp, Phi, chunk, split > 1 ? part : nullptr);
+    if (df) {
+        constexpr size_t smem = (size_t)NC * kTile * 12 + kStage * 12 * 4 + (size_t)kStage * NC * 8;
+        int* cexp = SG.cexp.as<int>();
+        NM_CUDA(cudaFuncSetAttribute(nbody_df_kernel<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        NM_CUDA(cudaMemsetAsync(cexp, 0, 64 * sizeof(int), s));
+        column_exp_kernel<<<(unsigned)std::min<int64_t>((np * b + 4095) / 4096, 1024), 256, 0, s>>>(np, b, Q, cexp);
+        count_launch();
+        nbody_df_kernel<NC><<<grid, kTile, smem, s>>>(np, SG.limbs.as<float>(), SG.inv_scale, invR, SG.G, Q, b, cexp,
+                                                      Phi, chunk, part);
+    } else {
+        nbody_kernel<NC><<<grid, kTile, 0, s>>>(np, SG.pts.as<double>(), invR, SG.G, Q, b, Phi, chunk, part);
+    }
     if (split > 1) {
         count_launch();
         const int64_t total = np * b;
         const int blocks = (int)std::min<int64_t>((total + 255) / 256, 4096);
-        nbody_reduce_kernel<<<blocks, 256, 0, s>>>(np, b, split, part, inv_R, G, Q, Phi);
+        nbody_reduce_kernel<<<blocks, 256, 0, s>>>(np, b, split, part, invR, SG.G, Q, Phi);
     }
     count_launch();
     NM_CUDA(cudaGetLastError());
@@ -522,8 +603,10 @@ int build_self_gravity(nm_problem* P, const double* xyz, const int32_t* tet, con
     return NM_OK;
 }
 
-// W -= C^T S C X for a block of b <= 64 columns (X, W row-major FP64).
-int apply_selfgrav(nm_problem* P, const double* X, int64_t ldx, double* W, int64_t ldw, int b, cudaStream_t s) {
+// W -= C^T S C X for a block of b <= 64 columns (X, W row-major FP64), the
+// sum over the points in double-float with df.
+int apply_selfgrav(nm_problem* P, const double* X, int64_t ldx, double* W, int64_t ldw, int b, bool df,
+                   cudaStream_t s) {
     SelfGravity& SG = P->sg;
     if (!SG.on) return NM_OK;
     if (b < 1 || b > 64) return fail(NM_EINVAL, "self-gravitation takes blocks of 1..64 columns");
@@ -535,15 +618,11 @@ int apply_selfgrav(nm_problem* P, const double* X, int64_t ldx, double* W, int64
     count_launch();
     NM_CUDA(cudaGetLastError());
     // the narrowest column group that holds the block (wider blocks: groups of 32)
-    const double *invR = SG.invR.as<double>(), *q = SG.q.as<double>();
-    const float* pts = SG.limbs.as<float>();
-    double *phi = SG.phi.as<double>(), *part = SG.part.as<double>();
-    if (nbody_cols(b) == 8)
-        NM_TRY(launch_nbody<8>(SG.np, pts, SG.inv_scale, invR, SG.G, q, b, SG.cexp.as<int>(), phi, part, s));
-    else if (nbody_cols(b) == 16)
-        NM_TRY(launch_nbody<16>(SG.np, pts, SG.inv_scale, invR, SG.G, q, b, SG.cexp.as<int>(), phi, part, s));
-    else
-        NM_TRY(launch_nbody<32>(SG.np, pts, SG.inv_scale, invR, SG.G, q, b, SG.cexp.as<int>(), phi, part, s));
+    switch (nbody_cols(b)) {
+        case 8: NM_TRY(launch_nbody<8>(SG, df, b, s)); break;
+        case 16: NM_TRY(launch_nbody<16>(SG, df, b, s)); break;
+        default: NM_TRY(launch_nbody<32>(SG, df, b, s));
+    }
     csr_spmm_kernel<<<(unsigned)((n + per - 1) / per), 256, 0, s>>>(
         n, SG.t_rp.as<int64_t>(), SG.t_col.as<int>(), SG.t_val.as<double>(), SG.phi.as<double>(), b, W, ldw, b, -1.0,
         1.0);

@@ -250,7 +250,7 @@ static int apply_K_t(nm_problem* P, const T* X, int64_t ldx, T* W, int64_t ldw, 
     }
     NM_TRY(launch_bsr33<T>(a, s));
     if (sg) {
-        NM_TRY(apply_selfgrav(P, (const double*)X, ldx, (double*)W, ldw, b, s));
+        NM_TRY(apply_selfgrav(P, (const double*)X, ldx, (double*)W, ldw, b, false, s));
         if (X1) NM_TRY(launch_dscale<T>(3, m.Nu, b, (T)inv_theta_M, m.dM, W, ldw, X1, b, s));
     }
     return NM_OK;
@@ -541,7 +541,7 @@ static int apply_K_mixed_core(nm_problem* P, const double* X, int64_t ldx, doubl
 static int apply_K_mixed(nm_problem* P, const double* X, int64_t ldx, double* W, int64_t ldw, int b, int k_P,
                          const MixScratch& S, cudaStream_t s, bool pre_split = false) {
     NM_TRY(apply_K_mixed_core(P, X, ldx, W, ldw, b, k_P, S, s, pre_split));
-    return apply_selfgrav(P, X, ldx, W, ldw, b, s);
+    return apply_selfgrav(P, X, ldx, W, ldw, b, P->use_df != 0, s);
 }
 
 static int apply_K_mixed_core(nm_problem* P, const double* X, int64_t ldx, double* W, int64_t ldw, int b,
