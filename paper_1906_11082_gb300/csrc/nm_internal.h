@@ -127,6 +127,7 @@ struct SelfGravity {
     DevBuf pts, invR;                 // double [3 np], [np]
     DevBuf limbs;                     // float [9 np]: the points in limbs (df_pair.cuh)
     double inv_scale = 1;             // their power-of-two scaling
+    bool df_ok = false;               // no two points too close for the limbs
     DevBuf cexp;                      // int [64]: exponents of the charge block's columns
     DevBuf c_rp, c_col, c_val;        // C: int64 [np + 1], int32, double
     DevBuf t_rp, t_col, t_val;        // C^T: int64 [n + 1], int32, double

@@ -305,6 +305,34 @@ __global__ void __launch_bounds__(kTile, 3) nbody_df_kernel(int64_t np, const fl
         if (c < nc) Phi[i * b + c0 + c] = G * fma(d, Q[i * b + c0 + c], sum(c));
 }
 
+// flag = 1 if the first limbs of two points come within 2^-19 of each other
+// (scaled coordinates). Closer pairs may lie below 2^-20, where the third limb
+// weighs enough for the dropped square of the low part to show (2^-50 of r^2
+// there, 2^-30 at 2^-30): the FP64 sums take such point sets.
+constexpr float kCloseSq = 0x1p-38f;
+__global__ void __launch_bounds__(kTile) close_points_kernel(int64_t np, const float* __restrict__ limbs, int* flag) {
+    __shared__ float sh[kTile][3];
+    const int64_t i = blockIdx.x * (int64_t)kTile + threadIdx.x;
+    float x[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) x[d] = i < np ? limbs[i * kLimbs + d] : 4.f;
+    float r2 = 4.f;
+    for (int64_t j0 = blockIdx.y * (int64_t)kTile; j0 < np; j0 += gridDim.y * (int64_t)kTile) {
+        const int64_t j = j0 + threadIdx.x;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) sh[threadIdx.x][d] = j < np ? limbs[j * kLimbs + d] : -4.f;
+        __syncthreads();
+        const int64_t self = i - j0;
+        for (int k = 0; k < kTile; ++k) {
+            const float dx = sh[k][0] - x[0], dy = sh[k][1] - x[1], dz = sh[k][2] - x[2];
+            const float q = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+            if (k != self) r2 = fminf(r2, q);
+        }
+        __syncthreads();
+    }
+    if (i < np && r2 < kCloseSq) atomicOr(flag, 1);
+}
+
 // Phi = G (sum over the source ranges of part + inv_R Q), ranges in order.
 __global__ void nbody_reduce_kernel(int64_t np, int b, int split, const double* __restrict__ part,
                                     const double* __restrict__ inv_R, double G, const double* __restrict__ Q,
@@ -585,7 +613,15 @@ int build_self_gravity(nm_problem* P, const double* xyz, const int32_t* tet, con
     split_points_kernel<<<1024, 256, 0, s>>>(np, 3, SG.pts.as<double>(), SG.inv_scale, SG.limbs.as<float>());
     count_launch();
     NM_CUDA(cudaGetLastError());
+    int* flag = SG.cexp.as<int>();   // free until the first product
+    int close = 0;
+    NM_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), s));
+    close_points_kernel<<<dim3((unsigned)((np + kTile - 1) / kTile), 8), kTile, 0, s>>>(np, SG.limbs.as<float>(), flag);
+    count_launch();
+    NM_CUDA(cudaGetLastError());
+    NM_CUDA(cudaMemcpyAsync(&close, flag, sizeof(int), cudaMemcpyDeviceToHost, s));
     NM_CUDA(cudaStreamSynchronize(s));
+    SG.df_ok = !close;
     std::vector<Entry> tr(ent.size());
     for (size_t k = 0; k < ent.size(); ++k) tr[k] = {ent[k].col, (int32_t)ent[k].row, ent[k].val};
     NM_TRY(upload_csr(ent, np, SG.c_rp, SG.c_col, SG.c_val, s));
@@ -604,7 +640,7 @@ int build_self_gravity(nm_problem* P, const double* xyz, const int32_t* tet, con
 }
 
 // W -= C^T S C X for a block of b <= 64 columns (X, W row-major FP64), the
-// sum over the points in double-float with df.
+// sum over the points in double-float with df where the points allow it.
 int apply_selfgrav(nm_problem* P, const double* X, int64_t ldx, double* W, int64_t ldw, int b, bool df,
                    cudaStream_t s) {
     SelfGravity& SG = P->sg;
@@ -612,6 +648,7 @@ int apply_selfgrav(nm_problem* P, const double* X, int64_t ldx, double* W, int64
     if (b < 1 || b > 64) return fail(NM_EINVAL, "self-gravitation takes blocks of 1..64 columns");
     const int64_t n = P->info.n;
     const int per = 256 / 32;
+    df = df && SG.df_ok;
     csr_spmm_kernel<<<(unsigned)((SG.np + per - 1) / per), 256, 0, s>>>(
         SG.np, SG.c_rp.as<int64_t>(), SG.c_col.as<int>(), SG.c_val.as<double>(), X, ldx, SG.q.as<double>(), b, b,
         1.0, 0.0);
