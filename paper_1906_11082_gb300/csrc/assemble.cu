@@ -441,8 +441,9 @@ __global__ void split_mass_kernel(int64_t n, const double* src, double inv, floa
 }
 
 // g(x_i) = -G sum_k m_k (x_i - r_k) / |x_i - r_k|^3 in FP64, sources staged in
-// shared memory: for meshes with edges below 2^-14 of their extent, whose pair
-// distances the limbs may not resolve
+// shared memory: for meshes of fewer than 16,384 tets, where it is the more
+// accurate form, and those with tets so flat that their barycentre comes too
+// close to a node for the limbs
 __global__ void __launch_bounds__(256) gravity_kernel(int64_t nx, const double* x, int64_t ns,
                                                       const double* src /* [ns][4]: r, m */,
                                                       double G, double* g) {
@@ -958,24 +959,35 @@ int assemble(nm_ctx* ctx, const nm_mesh* mesh, const nm_model* mdl, nm_problem* 
             DevBuf d_ux, d_src;
             NM_TRY(upload(d_ux, ux, s));
             NM_TRY(upload(d_src, src, s));
-            double far = 0, mmax = 0, emin = 1e300;
+            double far = 0, mmax = 0, near = 1e300;
             for (int d = 0; d < 3; ++d) far = std::max(far, std::max(std::fabs(lo[d]), std::fabs(hi[d])));
             for (int64_t t = 0; t < nt; ++t) {
                 mmax = std::max(mmax, src[4 * t + 3]);
-                for (int e = 0; e < 6; ++e) {
-                    const double* a = xyz + 3 * tet[4 * t + kEdge[e][0]];
-                    const double* b = xyz + 3 * tet[4 * t + kEdge[e][1]];
-                    const double dx = a[0] - b[0], dy = a[1] - b[1], dz = a[2] - b[2];
-                    emin = std::min(emin, dx * dx + dy * dy + dz * dz);
+                // A barycentre is a quarter of a height away from each face of
+                // its tet, and no node lies inside: the least distance of a
+                // pair, height = |det| / |cross product of the face|.
+                const double* x = &vx[12 * t];
+                double det = 0, cross2 = 0;
+                static const int kFace[4][3] = {{1, 2, 3}, {0, 2, 3}, {0, 1, 3}, {0, 1, 2}};
+                for (int f = 0; f < 4; ++f) {
+                    const double *p = x + 3 * kFace[f][0], *q = x + 3 * kFace[f][1], *r = x + 3 * kFace[f][2];
+                    const double u[3] = {q[0] - p[0], q[1] - p[1], q[2] - p[2]};
+                    const double v[3] = {r[0] - p[0], r[1] - p[1], r[2] - p[2]};
+                    const double n[3] = {u[1] * v[2] - u[2] * v[1], u[2] * v[0] - u[0] * v[2], u[0] * v[1] - u[1] * v[0]};
+                    cross2 = std::max(cross2, n[0] * n[0] + n[1] * n[1] + n[2] * n[2]);
+                    if (f == 3) det = std::fabs(n[0] * (x[9] - p[0]) + n[1] * (x[10] - p[1]) + n[2] * (x[11] - p[2]));
                 }
+                near = std::min(near, 0.25 * det / std::sqrt(cross2));
             }
             // powers of two: the scaling is exact
             const double S = std::exp2(std::ceil(std::log2(far))), M = std::exp2(std::ceil(std::log2(mmax)));
             // Double-float from 16,384 sources on: its error against quad
             // precision is 3e-15 to 4e-15 of |g| whatever their number, the
             // FP64 sum's 1.7e-15 at 1,980 sources and 7.6e-15 at 43,600 (one
-            // rounding of the running sum per source).
-            const bool df = nt >= 16384 && std::sqrt(emin) >= 0x1p-14 * S && S > 0x1p-200 && S < 0x1p200 &&
+            // rounding of the running sum per source). The limbs hold pairs
+            // from 2^-20 of the extent on (their dropped terms 2^-50 of r^2);
+            // 2^-16 is where edges of 2^-14 lie in a regular tet.
+            const bool df = nt >= 16384 && near >= 0x1p-16 * S && S > 0x1p-200 && S < 0x1p200 &&
                             M > 0x1p-400 && M < 0x1p400;
             DevBuf d_xl, d_sl, d_m;
             if (df) {

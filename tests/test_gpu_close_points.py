@@ -12,6 +12,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 from synth.model import layered_planet  # noqa: E402
+from oracle import fem  # noqa: E402
 
 
 @pytest.fixture(scope="module")
@@ -54,4 +55,28 @@ def test_mixed_self_gravitation_of_a_sliver(nm):
     P.apply_K(X, Z, k_P=40, prec=nm.NM_MIXED)
     assert bool(torch.isfinite(Z).all())
     assert float((Y - Z).abs().max() / Z.abs().max()) <= 1e-12
+    P.free()
+
+
+def test_reference_gravity_near_a_sliver(nm):
+    """Four points whose diagonals pass each other at t = 2^-28 + 2^-44 + 2^-46:
+    the barycentre is t / 2 from two mid-edge nodes, although no edge is short,
+    and rules the field there. Float triples would err by 2^-35 of it, with
+    18,000 other tets; FP64 sums agree to 1e-12, as for other meshes."""
+    t = 2.0 ** -28 + 2.0 ** -44 + 2.0 ** -46
+    c = np.array([0.5, 0.25, 0.25])
+    u, v = np.array([0.125, 0, 0]), np.array([0, 0.125, 0])
+    up = np.array([0, 0, t])
+    mesh, model = _with_tet(0.12, np.array([c + u, c - u, c + v + up, c - v + up]))
+    assert mesh.nt >= 16384
+    P = nm.Problem(nm.Context(0), mesh, model)
+    g = P.gravity()
+    tet, nv = mesh.tet.astype(np.int64), len(mesh.xyz)
+    pair = np.sort(np.stack([tet[:, list(e)] for e in ((0, 1), (0, 2), (0, 3), (1, 2), (1, 3), (2, 3))], 1), -1)
+    key = np.unique(pair[..., 0] * nv + pair[..., 1])
+    pos = np.concatenate([mesh.xyz, 0.5 * (mesh.xyz[key // nv] + mesh.xyz[key % nv])])[P.unodes()[1]]
+    near = np.flatnonzero(np.abs(pos - c).max(1) < 2.0 ** -20)
+    assert len(near) == 2
+    ref = fem.gravity_direct(pos[near], mesh.xyz, tet, model.rho, model.G)
+    assert np.abs(g[near] - ref).max() <= 1e-12 * np.abs(ref).max()
     P.free()
