@@ -398,12 +398,14 @@ struct MixScratch {
     float *w32, *xa, *xb, *xs, *es;
     float *Th, *Tl;   // double-float split of the block K_eff is applied to
     int ng = 1, bg = 0, bp = 0;
+    bool tma = false;   // the staged mass step (option "tma", blocks of 32 columns)
 };
 
 static int get_mix_scratch(nm_problem* P, int b, MixScratch& S) {
     const int64_t n = P->info.n, Np = P->info.Np;
     cluster_groups(b, &S.ng, &S.bg);
     S.bp = S.ng * S.bg;
+    S.tma = b == 32 && P->use_tma && P->Mr.tma_state == 1;
     // 16-byte aligned parts
     const int64_t nd = (n * b + 1) / 2 * 2, pd = (Np * b + 1) / 2 * 2, ng = (n * S.bg + 3) / 4 * 4, np = (n * S.bp + 3) / 4 * 4;
     const size_t need = (size_t)(3 * nd + 2 * pd) * sizeof(double) + (size_t)(5 * ng + 2 * np) * sizeof(float);
@@ -431,8 +433,9 @@ static int get_mix_scratch(nm_problem* P, int b, MixScratch& S) {
 
 // k steps of float Jacobi-Chebyshev semi-iteration for (A (x) I_R) x = w;
 // w, xa, xb, xout: (R nodes) x b floats with ld b, xout distinct from xa, xb.
+// tma: staged kernel for R = 3 (b = 32, tiles built).
 static int cheb32(nm_problem* P, const DevCSR& A, int R, int b, int k, double lo, double hi, const float* w,
-                  float* xa, float* xb, float* xout, cudaStream_t s, bool x1_ready = false) {
+                  float* xa, float* xb, float* xout, cudaStream_t s, bool x1_ready, bool tma) {
     const ChebCoef cc(lo, hi);
     const int64_t nodes = A.nrows;
     if (k == 1) return launch_dscale<float>(R, nodes, b, (float)cc.inv_theta, A.dinv32.as<float>(), w, b, xout, b, s);
@@ -466,7 +469,7 @@ static int cheb32(nm_problem* P, const DevCSR& A, int R, int b, int k, double lo
         a.ldn = b;
         a.om = (float)om;
         a.inv_theta = (float)cc.inv_theta;
-        if (R == 3 && b == 32 && P->use_tma && A.tma_state == 1) a.tma = A.tma;
+        if (R == 3 && tma) a.tma = A.tma;
         set_clusters(a, A, P);
         NM_TRY(launch_kron<float>(R, KRON_CHEB, a, s));
     }
@@ -489,7 +492,7 @@ static int mixed_solve(nm_problem* P, const DevCSR& A, int R, int bv, int k, con
     // S.es is free until the second solve writes it: the low part of W
     float* wl = df ? S.es : nullptr;
     NM_TRY(launch_convert_x1(R, A.nrows, b, bv, W, ldw, S.w32, wl, it, A.dinv32.as<float>(), fuse ? S.xa : nullptr, s));
-    NM_TRY(cheb32(P, A, R, b, k, kMassLo, kMassHi, S.w32, S.xa, S.xb, S.xs, s, fuse));
+    NM_TRY(cheb32(P, A, R, b, k, kMassLo, kMassHi, S.w32, S.xa, S.xb, S.xs, s, fuse, S.tma));
     bool x1 = false;
     if (df) {
         ResidDfArgs r;
@@ -511,7 +514,7 @@ static int mixed_solve(nm_problem* P, const DevCSR& A, int R, int bv, int k, con
         NM_TRY(launch_resid_mixed(R, A.nrows, A.rowptr.as<int>(), A.col.as<int>(), A.val.as<double>(), W, ldw,
                                   S.xs, S.w32, b, bv, s));
     }
-    return cheb32(P, A, R, b, k, kMassLo, kMassHi, S.w32, S.xa, S.xb, S.es, s, x1);
+    return cheb32(P, A, R, b, k, kMassLo, kMassHi, S.w32, S.xa, S.xb, S.es, s, x1, S.tma);
 }
 
 // The same for every column group of a block, each followed by its combine:

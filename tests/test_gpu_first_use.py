@@ -59,3 +59,20 @@ def test_first_float_product(nm, planet, first):
     assert rel_err(to_canonical(P, Y.double().cpu().numpy()), ref[first]) <= tol[first]
     assert rel_err(to_canonical(P, Z.double().cpu().numpy()), ref[second]) <= tol[second]
     P.free()
+
+
+@pytest.mark.parametrize("b", [30, 57, 64])
+def test_staged_step_leaves_other_widths_alone(nm, planet, b):
+    """Option tma is for blocks of 32 columns. Blocks that are padded to groups
+    of 32 give the same bits before and after a call that built its tiles."""
+    mesh, model, S = planet
+    P = nm.Problem(nm.Context(0), mesh, model)
+    P.set_option("tma", 1)
+    W = torch.randn((S.n, b), dtype=torch.float64, device=DEV)
+    W32 = torch.randn((S.n, 32), dtype=torch.float64, device=DEV)
+    X, Y, Y32 = torch.empty_like(W), torch.empty_like(W), torch.empty_like(W32)
+    P.solve_M(W, X, k_M=12, prec=nm.NM_MIXED)
+    P.solve_M(W32, Y32, k_M=12, prec=nm.NM_MIXED)
+    P.solve_M(W, Y, k_M=12, prec=nm.NM_MIXED)
+    assert bool((X == Y).all())
+    P.free()
