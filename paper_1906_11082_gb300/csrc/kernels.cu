@@ -951,14 +951,15 @@ int launch_resid_mixed(int R, int64_t nodes, const int* rowptr, const int* col, 
 }
 
 // N columns per thread (4, or 1 where widths or alignments do not allow the
-// vector accesses): 32-bit index arithmetic, the same operations per element.
-template <int N>
+// vector accesses), the same operations per element. I: index type, 32 bits
+// where the last stride past the end does not wrap.
+template <int N, typename I>
 __global__ void __launch_bounds__(kThreads) combine_kernel(const CombineArgs a) {
-    const unsigned nb = a.b / N, total = (unsigned)a.rows * nb;
+    const I nb = a.b / N, total = (I)a.rows * nb;
     const int dg = a.deg ? a.deg[0] + 1 : 0;
     const double* gt = a.gam_tab ? a.gam_tab + (int64_t)dg * a.gam_stride : nullptr;
-    for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
-        const unsigned i = t / nb;
+    for (I t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
+        const I i = t / nb;
         const int c = N * (int)(t - i * nb), cg = a.c0 + c;
         const int64_t ix = (int64_t)i * a.ldx + c, it = (int64_t)i * a.ldt + cg;
         float x[N], e[N];
@@ -1047,15 +1048,24 @@ int launch_inc_int(int* p, cudaStream_t s) {
     return NM_OK;
 }
 
+template <int N>
+static void combine_go(const CombineArgs& a, cudaStream_t s) {
+    const int64_t total = a.rows * a.b / N;
+    const unsigned grid = grid_for(total);
+    if (fits_u32(total, (int64_t)grid * kThreads))
+        combine_kernel<N, unsigned><<<grid, kThreads, 0, s>>>(a);
+    else
+        combine_kernel<N, uint64_t><<<grid, kThreads, 0, s>>>(a);
+}
+
 int launch_combine(const CombineArgs& a, cudaStream_t s) {
     if (a.rows * a.b == 0) return NM_OK;
-    if (a.rows * a.b > 0xFFFFFFFFll) return fail(NM_EINVAL, "block too large for the combine");
     const uintptr_t al = (uintptr_t)a.out | (uintptr_t)a.Tk | (uintptr_t)a.Tp | (uintptr_t)a.Tn | (uintptr_t)a.Z |
                          (uintptr_t)a.x32 | (uintptr_t)a.e32 | (uintptr_t)a.Th | (uintptr_t)a.Tl;
     if (((a.b | a.c0) & 3) == 0 && ((a.ldx | a.ldh) & 3) == 0 && ((a.ldt | a.ldz) & 1) == 0 && (al & 15) == 0)
-        combine_kernel<4><<<grid_for(a.rows * a.b / 4), kThreads, 0, s>>>(a);
+        combine_go<4>(a, s);
     else
-        combine_kernel<1><<<grid_for(a.rows * a.b), kThreads, 0, s>>>(a);
+        combine_go<1>(a, s);
     count_launch();
     NM_CUDA(cudaGetLastError());
     return NM_OK;

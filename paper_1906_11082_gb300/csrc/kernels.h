@@ -10,6 +10,11 @@ namespace nm {
 void count_launch(uint64_t n = 1);
 uint64_t launches_so_far();
 
+// Whether a grid-stride loop over total elements may count in 32 bits: its
+// counter, at most total - 1 before the last addition of the stride, must not
+// wrap to a value below total.
+inline bool fits_u32(int64_t total, int64_t stride) { return total + stride <= 0xFFFFFFFFll; }
+
 enum KronMode { KRON_PLAIN = 0, KRON_CHEB = 1, KRON_CHEB_FILT = 2, KRON_CORI = 3 };
 
 // Row tiles of a scalar CSR matrix for the bulk-copy staged mass step
