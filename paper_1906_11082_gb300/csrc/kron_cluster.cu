@@ -27,7 +27,9 @@
 // b = 32: 298 -> 234 us, pressure rows (82k) 46 -> 26 us. 199k dof: b = 16
 // 55 -> 23 us, b = 64 199 -> 89 us (were per-lane scalar gathers).
 #include <algorithm>
+#include <atomic>
 #include <cstdint>
+#include <new>
 #include <vector>
 
 #include "kernels.h"
@@ -364,9 +366,7 @@ __global__ void cluster_values_kernel(int64_t n4, const int* at, const float* va
 // Clusters inside windows of kMaxRows consecutive (Morton) rows, greedily: the
 // undone row with most entries takes the three rows that add fewest new
 // columns for the columns they share.
-int build_clusters(DevCSR& A, cudaStream_t s) {
-    if (A.cl_state) return NM_OK;
-    A.cl_state = -1;
+static int make_clusters(DevCSR& A, cudaStream_t s) {
     const int64_t N = A.nrows;
     if (N < 1 || A.nnz < 1) return NM_OK;
     const int64_t nwin = (N + kMaxRows - 1) / kMaxRows;
@@ -379,76 +379,82 @@ int build_clusters(DevCSR& A, cudaStream_t s) {
     std::vector<Win> win(nwin);
     const int* rp = A.h_rowptr.data();
     const int* col = A.h_col.data();
+    std::atomic<bool> no_memory{false};   // an exception must not leave the parallel region
 #pragma omp parallel
     {
         std::vector<int> cols, pos;
         std::vector<uint64_t> bits, cur;
 #pragma omp for schedule(dynamic, 32)
         for (int64_t w = 0; w < nwin; ++w) {
-            const int r0 = (int)(w * kMaxRows), n = (int)std::min<int64_t>(kMaxRows, N - r0);
-            cols.assign(col + rp[r0], col + rp[r0 + n]);
-            std::sort(cols.begin(), cols.end());
-            cols.erase(std::unique(cols.begin(), cols.end()), cols.end());
-            const int U = (int)cols.size(), words = (U + 63) / 64;
-            bits.assign((size_t)n * words, 0);
-            cur.assign(words, 0);
-            pos.assign((size_t)n * U, -1);
-            for (int i = 0; i < n; ++i)
-                for (int e = rp[r0 + i]; e < rp[r0 + i + 1]; ++e) {
-                    const int l = (int)(std::lower_bound(cols.begin(), cols.end(), col[e]) - cols.begin());
-                    bits[(size_t)i * words + l / 64] |= 1ull << (l % 64);
-                    pos[(size_t)i * U + l] = e;
-                }
-            int ord[kMaxRows];
-            bool done[kMaxRows] = {};
-            for (int i = 0; i < n; ++i) ord[i] = i;
-            std::sort(ord, ord + n, [&](int x, int y) {
-                const int dx = rp[r0 + x + 1] - rp[r0 + x], dy = rp[r0 + y + 1] - rp[r0 + y];
-                return dx != dy ? dx > dy : x < y;
-            });
-            int64_t c = w * kPer;
-            for (int o = 0; o < n; ++o) {
-                const int seed = ord[o];
-                if (done[seed]) continue;
-                int m[4] = {seed, -1, -1, -1};
-                done[seed] = true;
-                for (int k = 0; k < words; ++k) cur[k] = bits[(size_t)seed * words + k];
-                for (int f = 1; f < 4; ++f) {
-                    int best = -1, bs = 1 << 30;
-                    for (int i = 0; i < n; ++i) {
-                        if (done[i]) continue;
-                        int grow = 0, shared = 0;
-                        for (int k = 0; k < words; ++k) {
-                            const uint64_t b = bits[(size_t)i * words + k];
-                            grow += __builtin_popcountll(b & ~cur[k]);
-                            shared += __builtin_popcountll(b & cur[k]);
-                        }
-                        if (2 * grow - shared < bs) {
-                            bs = 2 * grow - shared;
-                            best = i;
-                        }
+            try {
+                const int r0 = (int)(w * kMaxRows), n = (int)std::min<int64_t>(kMaxRows, N - r0);
+                cols.assign(col + rp[r0], col + rp[r0 + n]);
+                std::sort(cols.begin(), cols.end());
+                cols.erase(std::unique(cols.begin(), cols.end()), cols.end());
+                const int U = (int)cols.size(), words = (U + 63) / 64;
+                bits.assign((size_t)n * words, 0);
+                cur.assign(words, 0);
+                pos.assign((size_t)n * U, -1);
+                for (int i = 0; i < n; ++i)
+                    for (int e = rp[r0 + i]; e < rp[r0 + i + 1]; ++e) {
+                        const int l = (int)(std::lower_bound(cols.begin(), cols.end(), col[e]) - cols.begin());
+                        bits[(size_t)i * words + l / 64] |= 1ull << (l % 64);
+                        pos[(size_t)i * U + l] = e;
                     }
-                    if (best < 0) break;
-                    m[f] = best;
-                    done[best] = true;
-                    for (int k = 0; k < words; ++k) cur[k] |= bits[(size_t)best * words + k];
+                int ord[kMaxRows];
+                bool done[kMaxRows] = {};
+                for (int i = 0; i < n; ++i) ord[i] = i;
+                std::sort(ord, ord + n, [&](int x, int y) {
+                    const int dx = rp[r0 + x + 1] - rp[r0 + x], dy = rp[r0 + y + 1] - rp[r0 + y];
+                    return dx != dy ? dx > dy : x < y;
+                });
+                int64_t c = w * kPer;
+                for (int o = 0; o < n; ++o) {
+                    const int seed = ord[o];
+                    if (done[seed]) continue;
+                    int m[4] = {seed, -1, -1, -1};
+                    done[seed] = true;
+                    for (int k = 0; k < words; ++k) cur[k] = bits[(size_t)seed * words + k];
+                    for (int f = 1; f < 4; ++f) {
+                        int best = -1, bs = 1 << 30;
+                        for (int i = 0; i < n; ++i) {
+                            if (done[i]) continue;
+                            int grow = 0, shared = 0;
+                            for (int k = 0; k < words; ++k) {
+                                const uint64_t b = bits[(size_t)i * words + k];
+                                grow += __builtin_popcountll(b & ~cur[k]);
+                                shared += __builtin_popcountll(b & cur[k]);
+                            }
+                            if (2 * grow - shared < bs) {
+                                bs = 2 * grow - shared;
+                                best = i;
+                            }
+                        }
+                        if (best < 0) break;
+                        m[f] = best;
+                        done[best] = true;
+                        for (int k = 0; k < words; ++k) cur[k] |= bits[(size_t)best * words + k];
+                    }
+                    int u = 0;
+                    for (int l = 0; l < U; ++l) {
+                        if (!((cur[l / 64] >> (l % 64)) & 1)) continue;
+                        for (int f = 0; f < 4; ++f) win[w].at.push_back(m[f] < 0 ? -1 : pos[(size_t)m[f] * U + l]);
+                        win[w].col.push_back(cols[l]);
+                        ++u;
+                    }
+                    for (; u % kPad; ++u) {
+                        for (int f = 0; f < 4; ++f) win[w].at.push_back(-1);
+                        win[w].col.push_back(win[w].col.back());
+                    }
+                    for (int f = 0; f < 4; ++f) rows[4 * c + f] = m[f] < 0 ? -1 : r0 + m[f];
+                    ptr[++c] = u;
                 }
-                int u = 0;
-                for (int l = 0; l < U; ++l) {
-                    if (!((cur[l / 64] >> (l % 64)) & 1)) continue;
-                    for (int f = 0; f < 4; ++f) win[w].at.push_back(m[f] < 0 ? -1 : pos[(size_t)m[f] * U + l]);
-                    win[w].col.push_back(cols[l]);
-                    ++u;
-                }
-                for (; u % kPad; ++u) {
-                    for (int f = 0; f < 4; ++f) win[w].at.push_back(-1);
-                    win[w].col.push_back(win[w].col.back());
-                }
-                for (int f = 0; f < 4; ++f) rows[4 * c + f] = m[f] < 0 ? -1 : r0 + m[f];
-                ptr[++c] = u;
+            } catch (const std::bad_alloc&) {
+                no_memory = true;
             }
         }
     }
+    if (no_memory) throw std::bad_alloc();
     int64_t ne = 0;
     for (int64_t c = 0; c < ncl; ++c) {
         ne += ptr[c + 1];
@@ -464,8 +470,7 @@ int build_clusters(DevCSR& A, cudaStream_t s) {
     DevBuf at;
     auto up = [&](DevBuf& b, const void* src, size_t bytes) -> int {
         NM_TRY(b.alloc(bytes));
-        NM_CUDA(cudaMemcpyAsync(b.p, src, bytes, cudaMemcpyHostToDevice, s));
-        return NM_OK;
+        return copy_in(b.p, src, bytes, s);
     };
     NM_TRY(up(at, fa.data(), fa.size() * sizeof(int)));
     NM_TRY(up(A.cl_ptr, ptr.data(), ptr.size() * sizeof(int)));
@@ -476,7 +481,7 @@ int build_clusters(DevCSR& A, cudaStream_t s) {
         4 * ne, at.as<int>(), A.val32.as<float>(), A.cl_val.as<float>());
     count_launch();
     NM_CUDA(cudaGetLastError());
-    NM_CUDA(cudaStreamSynchronize(s));   // the host vectors and the positions are released here
+    NM_CUDA(cudaStreamSynchronize(s));   // the positions are released here, later calls may come on another stream
     int dev = 0;
     NM_CUDA(cudaGetDevice(&dev));
     NM_CUDA(cudaDeviceGetAttribute(&A.cl.sms, cudaDevAttrMultiProcessorCount, dev));
@@ -487,6 +492,20 @@ int build_clusters(DevCSR& A, cudaStream_t s) {
     A.cl.rows = A.cl_rows.as<int4>();
     A.cl_state = 1;
     return NM_OK;
+}
+
+// State -1 only for matrices without clusters: a call that finds no memory
+// fails, and the next one tries again.
+int build_clusters(DevCSR& A, cudaStream_t s) {
+    if (A.cl_state) return NM_OK;
+    int rc;
+    try {
+        rc = make_clusters(A, s);
+    } catch (const std::bad_alloc&) {
+        rc = fail(NM_ENOMEM, "host allocation failed");
+    }
+    if (rc == NM_OK && A.cl_state == 0) A.cl_state = -1;
+    return rc;
 }
 
 }  // namespace nm
