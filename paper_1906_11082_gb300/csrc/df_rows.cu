@@ -23,7 +23,6 @@
 // dof, 32 columns 723 -> 662 us, 199k dof, 64 columns 332 -> 236 us. They take
 // w as a pair of floats: subtracting in double held the FP64 pipe for 0.3 ms.
 #include <algorithm>
-#include <atomic>
 #include <cstdint>
 
 #include "kernels.h"
@@ -312,19 +311,6 @@ __global__ void __launch_bounds__(kThreads) resid_df_rows_kernel(const ResidDfAr
 
 // ----------------------------------------------------------------- launches
 namespace {
-
-int sm_count() {
-    static std::atomic<int> n{0};
-    int v = n.load(std::memory_order_relaxed);
-    if (v == 0) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1)
-            v = 148;
-        n.store(v, std::memory_order_relaxed);
-    }
-    return v;
-}
 
 template <int L, int S>
 unsigned blocks(int nrows) {

@@ -888,63 +888,44 @@ __device__ __forceinline__ void store_n(double* p, const double* v) {
     }
 }
 
-template <int R, int CPT>
+template <int R>
 __global__ void __launch_bounds__(kThreads) resid_mixed_kernel(int64_t nodes, const int* __restrict__ rowptr,
                                                                const int* __restrict__ col,
                                                                const double* __restrict__ val,
                                                                const double* __restrict__ W, int64_t ldw,
                                                                const float* __restrict__ x, float* r, int b, int bv,
                                                                int tpr_shift) {
-    const int tpr = 1 << tpr_shift;
-    const int lane = threadIdx.x & (tpr - 1);
+    const int c = threadIdx.x & ((1 << tpr_shift) - 1);
     const int64_t row = (int64_t)blockIdx.x * (kThreads >> tpr_shift) + (threadIdx.x >> tpr_shift);
-    if (row >= nodes) return;
-    double acc[CPT][R];
+    if (row >= nodes || c >= b) return;
+    double acc[R];
 #pragma unroll
-    for (int q = 0; q < CPT; ++q)
-#pragma unroll
-        for (int k = 0; k < R; ++k) acc[q][k] = 0.0;
+    for (int k = 0; k < R; ++k) acc[k] = 0.0;
     const int e0 = __ldg(rowptr + row), e1 = __ldg(rowptr + row + 1);
     for (int e = e0; e < e1; ++e) {
         const int64_t j = __ldg(col + e);
         const double v = __ldg(val + e);
-        const float* xj = x + (int64_t)R * j * b;
+        const float* xj = x + (int64_t)R * j * b + c;
 #pragma unroll
-        for (int q = 0; q < CPT; ++q) {
-            const int c = lane + q * tpr;
-            if (c < b) {
-#pragma unroll
-                for (int k = 0; k < R; ++k) acc[q][k] += v * (double)__ldg(xj + k * b + c);
-            }
-        }
+        for (int k = 0; k < R; ++k) acc[k] += v * (double)__ldg(xj + k * b);
     }
 #pragma unroll
-    for (int q = 0; q < CPT; ++q) {
-        const int c = lane + q * tpr;
-        if (c >= b) continue;
-#pragma unroll
-        for (int k = 0; k < R; ++k) {
-            const int64_t rr = R * row + k;
-            r[rr * b + c] = (float)((c < bv ? W[rr * ldw + c] : 0.0) - acc[q][k]);
-        }
+    for (int k = 0; k < R; ++k) {
+        const int64_t rr = R * row + k;
+        r[rr * b + c] = (float)((c < bv ? W[rr * ldw + c] : 0.0) - acc[k]);
     }
 }
 
 int launch_resid_mixed(int R, int64_t nodes, const int* rowptr, const int* col, const double* val,
                        const double* W, int64_t ldw, const float* x32, float* r32, int b, int bv, cudaStream_t s) {
-    if (b < 1 || b > 64) return fail(NM_EINVAL, "block width must be in 1..64");
+    if (b < 1 || b > 32) return fail(NM_EINVAL, "residual blocks are 1 .. 32 columns wide");
     const int shift = tpr_shift_for(b);
-    const int cpt = (b + (1 << shift) - 1) >> shift;
     const int64_t grid = (nodes + (kThreads >> shift) - 1) / (kThreads >> shift);
     if (grid == 0) return NM_OK;
-    if (R == 3 && cpt == 1)
-        resid_mixed_kernel<3, 1><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, val, W, ldw, x32, r32, b, bv, shift);
-    else if (R == 3)
-        resid_mixed_kernel<3, 2><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, val, W, ldw, x32, r32, b, bv, shift);
-    else if (cpt == 1)
-        resid_mixed_kernel<1, 1><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, val, W, ldw, x32, r32, b, bv, shift);
+    if (R == 3)
+        resid_mixed_kernel<3><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, val, W, ldw, x32, r32, b, bv, shift);
     else
-        resid_mixed_kernel<1, 2><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, val, W, ldw, x32, r32, b, bv, shift);
+        resid_mixed_kernel<1><<<(unsigned)grid, kThreads, 0, s>>>(nodes, rowptr, col, val, W, ldw, x32, r32, b, bv, shift);
     count_launch();
     NM_CUDA(cudaGetLastError());
     return NM_OK;

@@ -184,8 +184,8 @@ int launch_dscale(int R, int64_t nodes, int b, T inv_theta, const T* dinv, const
 
 // r32 = float(W - (A (x) I_R) x32) with double matrix values and double
 // sums over the float iterate (the refinement residual of a mixed solve).
-// x32, r32 dense (ld b); W holds the first bv of the b columns (the others
-// count as zero).
+// x32, r32 dense (ld b, at most 32); W holds the first bv of the b columns (the
+// others count as zero).
 int launch_resid_mixed(int R, int64_t nodes, const int* rowptr, const int* col, const double* val,
                        const double* W, int64_t ldw, const float* x32, float* r32, int b, int bv, cudaStream_t s);
 

@@ -13,7 +13,8 @@
 // f32x2), half the gathered bytes.
 //
 // Layout: S lane groups of L = (columns / 4) lanes split a cluster's entries,
-// U = 3 entries' records are in flight per lane, entries are padded to S U.
+// U = 3 entries' records are in flight per lane, entries are padded to a
+// multiple of six (S U for two groups; four groups skip what lies past the end).
 // Warps walk clusters with a grid stride (one wave), the next cluster's header
 // and first columns being fetched during the current one, so no chain of
 // dependent loads is exposed between clusters; the epilogue's streams are

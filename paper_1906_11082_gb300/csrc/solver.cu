@@ -670,12 +670,8 @@ static int filter_apply_mixed(nm_problem* P, const nm_filter* f, const double* Y
     NM_TRY(launch_scale_copy<double>(n, b, 1.0, Y, ldy, S.TA, b, s));
     // launches of one K_eff product and of one mass solve with its combine
     const int64_t per_k = 2 * (f->k_M - 1) + 3, kl = 1 + (P->info.Np > 0 ? 1 + S.ng * (2 * (f->k_P - 1) + 3) : 0);
-    // the padding columns of the split block stay zero: the combines write
-    // the block's own columns only
-    if (P->use_df && S.bp > b && d > 1) {
-        NM_CUDA(cudaMemsetAsync(S.Th, 0, (size_t)n * S.bp * sizeof(float), s));
-        NM_CUDA(cudaMemsetAsync(S.Tl, 0, (size_t)n * S.bp * sizeof(float), s));
-    }
+    // The padding columns of the split block are zero from degree 0 on, whose
+    // split writes them: the combines write the block's own columns only.
     // One degree k of the recurrence (T_k in cur, T_{k-1} in prev; T_{k+1}
     // overwrites prev). With dev_gam the combine takes gamma_{k+1} from the
     // device table at the device-side degree counter (graph replay).
