@@ -55,9 +55,10 @@ enum {
 
 /* NM_F64: every step in double. NM_F32: the whole filter recurrence in
  * float. NM_MIXED: double recurrence and K_eff SpMMs; each inner solve (mass
- * and fluid pressure) is k steps of float semi-iteration, one double
- * residual r = w - A x (float iterate, double values and sums), and k more
- * float steps on r, so the applied inverse is accurate to ~(2 rho^k)^2
+ * and fluid pressure) is k steps of float semi-iteration, one residual
+ * r = w - A x of the float iterate, and k more float steps on r; products and
+ * residual run in double-float (about 48 bits: values, w and sums as pairs of
+ * floats) or, with the option "double_float" at 0, in double, so the applied inverse is accurate to ~(2 rho^k)^2
  * while its vectors carry double rounding only. Blocks are double. */
 typedef enum { NM_F64 = 0, NM_F32 = 1, NM_MIXED = 2 } nm_prec;
 typedef enum { NM_UNIT_OMEGA = 0, NM_UNIT_OMEGA2 = 1 } nm_unit;

@@ -381,9 +381,11 @@ __global__ void face_kernel(const FaceArgs A) {
 // (df_pair.cuh): about 100 float operations a pair. Each run of 8 sources is
 // summed in double-float and added in FP64 (its own rounding, 2^-47 of the
 // run's sum, averages out over the runs). Targets x and sources src as limbs,
-// masses as (hi, lo) pairs. Bound by the float pipe: 66,309 x 43,600 pairs at
-// 101 operations take 7.8 ms at its peak, measured 12.4 ms; the FP64 form below
-// (21 FP64 operations a pair) takes 103 ms.
+// masses as (hi, lo) pairs. Bound by instruction issue (71% busy; the float pipe
+// 60%, the FP64 pipe of the runs' additions 57%) with 12 warps per SM: 66,309 x
+// 43,600 pairs at 101 operations take 7.8 ms at the float pipe's peak, measured
+// 12.4 ms (14.1 ms alone under a profiler); the FP64 form below (21 FP64
+// operations a pair) takes 103 ms.
 constexpr int kGravTile = 128, kGravRun = 8;
 __global__ void __launch_bounds__(kGravTile) gravity_df_kernel(int64_t nx, const float* __restrict__ x, int64_t ns,
                                                               const float* __restrict__ src,
@@ -982,9 +984,10 @@ int assemble(nm_ctx* ctx, const nm_mesh* mesh, const nm_model* mdl, nm_problem* 
             // powers of two: the scaling is exact
             const double S = std::exp2(std::ceil(std::log2(far))), M = std::exp2(std::ceil(std::log2(mmax)));
             // Double-float from 16,384 sources on: its error against quad
-            // precision is 3e-15 to 4e-15 of |g| whatever their number, the
-            // FP64 sum's 1.7e-15 at 1,980 sources and 7.6e-15 at 43,600 (one
-            // rounding of the running sum per source). The limbs hold pairs
+            // precision (root mean square) is 3.2e-15 of |g| at 16,400 sources,
+            // 3.8e-15 at 43,600 and 5.2e-15 at 106,000, the FP64 sum's 5.1e-15,
+            // 8.3e-15 and 1.0e-14 (one rounding of the running sum per source),
+            // and 1.7e-15 at 1,980. The limbs hold pairs
             // from 2^-20 of the extent on (their dropped terms 2^-50 of r^2);
             // 2^-16 is where edges of 2^-14 lie in a regular tet.
             const bool df = nt >= 16384 && near >= 0x1p-16 * S && S > 0x1p-200 && S < 0x1p200 &&

@@ -21,7 +21,9 @@
 // columns 75 -> 36 us.
 // The residuals are bound by their gathers (three entries in flight): 1.15M
 // dof, 32 columns 723 -> 662 us, 199k dof, 64 columns 332 -> 236 us. They take
-// w as a pair of floats: subtracting in double held the FP64 pipe for 0.3 ms.
+// w as a pair of floats (48 bits): subtracting in double held the FP64 pipe for
+// 0.3 ms, and taking w exactly (three floats) changes no error: solves, products
+// and filters of 4k to 1.15M dof at 18 to 40 inner steps within 1% of each other.
 #include <algorithm>
 #include <cstdint>
 

@@ -25,8 +25,10 @@
 // serial phases), per-thread cp.async rings 349 us.
 //
 // Per step, 1.15M dof, before (one row per warp, 16-byte lane groups) and now:
-// b = 32: 298 -> 234 us, pressure rows (82k) 46 -> 26 us. 199k dof: b = 16
-// 55 -> 23 us, b = 64 199 -> 89 us (were per-lane scalar gathers).
+// b = 32: 298 -> 239 us, pressure rows (82k) 46 -> 23 us in a chain of steps (34
+// us with cold caches). 199k dof: b = 16 55 -> 23 us, b = 64 199 -> 89 us (were
+// per-lane scalar gathers). The clusters are built on the host at the first
+// float or mixed call: with the float copies 11 ms at 199k dof, 52 ms at 1.15M.
 #include <algorithm>
 #include <atomic>
 #include <cstdint>

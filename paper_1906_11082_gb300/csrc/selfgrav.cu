@@ -210,8 +210,9 @@ __device__ __forceinline__ double up_scale(int e) { return e < 1 || e > 2045 ? 1
 // (root mean square), by 1.3e-15 to 2.9e-15 with nbody_kernel; that of charges
 // of one sign by 3e-16 to 1.3e-15 against 1.0e-15 to 1.2e-15, whose 1/r is
 // biased. Hence the mixed form only, whose option "double_float" chooses.
-// Bound by the float pipe: 36,160 points, 32 columns, 444 operations a pair
-// take 15.5 ms at its peak; measured 25 ms.
+// Bound by instruction issue (77% busy, the float pipe 65%): 36,160 points, 32
+// columns, 444 float operations a pair take 15.5 ms at that pipe's peak;
+// measured 25 ms.
 template <int NC>
 __global__ void __launch_bounds__(kTile, 3) nbody_df_kernel(int64_t np, const float* __restrict__ pts, double scale,
                                                      const double* __restrict__ inv_R, double G,
