@@ -84,8 +84,8 @@ SERVING_SLICES = [(4.0, 5.5), (4.5, 6.0), (3.5, 5.0)]
 # and the SHA-256 of kron_cluster.cu when it was taken: once the kernel source
 # changes the figure no longer describes it and the bench reports traffic
 # null.
-TRAFFIC_CAPTURE = {"kernel": "kron_cluster_kernel<3, 8>", "bytes": 570_886_784 + 124_145_664,
-                   "kernel_sha256": "25da5ade7a2f24bf627739e814e1db7ded87261c26b555f17135624c22b99292"}
+TRAFFIC_CAPTURE = {"kernel": "kron_cluster_kernel<3, 8>", "bytes": 570_759_040 + 124_194_816,
+                   "kernel_sha256": "76ca7364a04cafa270e6bede9f5e29d22b8e1c661f3c1b34d666548a16b60f29"}
 
 # FP64 peak of GB300 (NVIDIA's published B300 figure, 1.25 TFLOP/s; equal to
 # 152 SMs x ~2.05 GHz x 2 FP64 FMA per SM per clock x 2 flop).
