@@ -30,7 +30,9 @@
  *  - Streams: calls that take a cudaStream_t (passed as void*) only
  *    enqueue work on it; NULL means the legacy default stream. Calls
  *    without a stream argument (assembly, lanczos_slice, ritz) run on the
- *    problem's own stream and return after synchronising it.
+ *    problem's own stream and return after synchronising it; that stream
+ *    does not wait for others, so what they read from the device (a basis,
+ *    a start block) and earlier calls on the problem have to be complete.
  *  - Precision: NM_F64 computes in double, NM_F32 in float (values and
  *    accumulators), for the filter-path calls that take an nm_prec.
  */

@@ -161,6 +161,17 @@ def _dptr(t):
     return C.c_void_p(t.data_ptr())
 
 
+def _ready(t):
+    """Device pointer of an input of a call that runs on the library's own
+    stream, once the work queued on the current stream has made it (or None)."""
+    if t is None:
+        return None
+    if t.is_cuda:
+        import torch
+        torch.cuda.current_stream(t.device).synchronize()
+    return C.c_void_p(t.data_ptr())
+
+
 def _stream(stream):
     if stream is None:
         import torch
@@ -258,6 +269,7 @@ class Result:
             p = _lib.nm_result_vectors(self.h)
             torch.cuda.synchronize()
             _memcpy_d2d(out.data_ptr(), p, n * k * (16 if cplx else 8))
+            torch.cuda.synchronize()   # the copy is on the legacy stream, the caller may use another
         return out
 
     def free(self):
@@ -405,7 +417,7 @@ class Problem:
     def lanczos_slice(self, block, degree, k_M=0, k_P=0, max_blocks=40, check_every=1, prec=NM_F64,
                       tol=1e-6, seed=1, start=None, bounds_steps=40, allow_unconverged=False, log_every=0):
         o = nm_slice_opts(block, degree, k_M, k_P, max_blocks, check_every, prec, tol, seed,
-                          C.c_void_p(start.data_ptr()) if start is not None else None, bounds_steps, log_every)
+                          _ready(start), bounds_steps, log_every)
         h = C.c_void_p()
         rc = _lib.nm_lanczos_slice(self.h, C.byref(o), C.byref(h))
         if rc != NM_OK and not (rc == NM_ENOTCONV and h.value and allow_unconverged):
@@ -438,7 +450,7 @@ class Problem:
         """Begin a resumable filtered block Lanczos run (nm_lanczos_begin):
         slices=None solves the interval of set_interval, else [(lo, hi), ...]."""
         o = nm_slice_opts(block, degree, k_M, k_P, max_blocks, check_every, prec, tol, seed,
-                          C.c_void_p(start.data_ptr()) if start is not None else None, bounds_steps, log_every)
+                          _ready(start), bounds_steps, log_every)
         if slices is None:
             S, lo, hi = 0, None, None
         else:
@@ -454,7 +466,8 @@ class Problem:
         m = V.shape[1]
         le = None if lam_e is None else np.ascontiguousarray(lam_e, np.float64)
         h = C.c_void_p()
-        _check(_lib.nm_ritz(self.h, mode, _dptr(V), V.stride(0), m,
+        _dptr(V)
+        _check(_lib.nm_ritz(self.h, mode, _ready(V), V.stride(0), m,
                             le.ctypes.data_as(C.c_void_p) if le is not None else None, C.byref(h)), self.ctx.h)
         return Result(self.ctx, h)
 
@@ -514,8 +527,7 @@ class LanczosRun:
     def add(self, lo, hi, unit=NM_UNIT_OMEGA, seed=1, start=None):
         """A slice joins the running batch; returns its slice number."""
         idx = C.c_int()
-        _check(_lib.nm_lanczos_add(self.h, lo, hi, unit, seed, C.c_void_p(start.data_ptr()) if start is not None
-                                   else None, C.byref(idx)), self.prob.ctx.h)
+        _check(_lib.nm_lanczos_add(self.h, lo, hi, unit, seed, _ready(start), C.byref(idx)), self.prob.ctx.h)
         self.nslices = max(self.nslices, idx.value + 1)
         return idx.value
 
