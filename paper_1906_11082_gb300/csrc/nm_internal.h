@@ -124,9 +124,9 @@ struct SelfGravity {
     int on = 0;
     int64_t np = 0;
     double G = 0;
-    DevBuf pts, invR;                 // double [3 np], [np]
+    DevBuf pts, invR;                 // double [3 np] (scaled by inv_scale), [np]
     DevBuf limbs;                     // float [9 np]: the points in limbs (df_pair.cuh)
-    double inv_scale = 1;             // their power-of-two scaling
+    double inv_scale = 1;             // power of two that brings the points to [-1, 1]
     bool df_ok = false;               // no two points too close for the limbs
     DevBuf cexp;                      // int [64]: exponents of the charge block's columns
     DevBuf c_rp, c_col, c_val;        // C: int64 [np + 1], int32, double

@@ -122,9 +122,11 @@ __device__ __forceinline__ double inv_dist(double r2) {
 // memory kTile at a time. With split > 1 (small point sets, to fill the
 // machine) CTA z sums the sources of its range [z chunk, (z + 1) chunk) into
 // part[z] and nbody_reduce_kernel adds the ranges in order. Bound by the FP64
-// pipe: 36,160 points, 32 columns 98 ms.
+// pipe: 36,160 points, 32 columns 98 ms. pts are scaled by the power of two
+// scale, so that the float estimate neither overflows nor underflows in any
+// units; the sums are scaled back exactly.
 template <int NC>
-__global__ void __launch_bounds__(kTile) nbody_kernel(int64_t np, const double* __restrict__ pts,
+__global__ void __launch_bounds__(kTile) nbody_kernel(int64_t np, const double* __restrict__ pts, double scale,
                                                      const double* __restrict__ inv_R, double G,
                                                      const double* __restrict__ Q, int b, double* Phi,
                                                      int64_t chunk, double* part) {
@@ -165,6 +167,8 @@ __global__ void __launch_bounds__(kTile) nbody_kernel(int64_t np, const double* 
         __syncthreads();
     }
     if (i >= np) return;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) acc[c] *= scale;
     if (part) {
         double* o = part + ((int64_t)blockIdx.z * np + i) * b + c0;
 #pragma unroll
@@ -386,7 +390,7 @@ int launch_nbody(SelfGravity& SG, bool df, int b, cudaStream_t s) {
         nbody_df_kernel<NC><<<grid, kTile, smem, s>>>(np, SG.limbs.as<float>(), SG.inv_scale, invR, SG.G, Q, b, cexp,
                                                       Phi, chunk, part);
     } else {
-        nbody_kernel<NC><<<grid, kTile, 0, s>>>(np, SG.pts.as<double>(), invR, SG.G, Q, b, Phi, chunk, part);
+        nbody_kernel<NC><<<grid, kTile, 0, s>>>(np, SG.pts.as<double>(), SG.inv_scale, invR, SG.G, Q, b, Phi, chunk, part);
     }
     if (split > 1) {
         count_launch();
@@ -603,15 +607,16 @@ int build_self_gravity(nm_problem* P, const double* xyz, const int32_t* tet, con
     NM_TRY(SG.pts.alloc(pts.size() * sizeof(double)));
     NM_TRY(SG.invR.alloc(invR.size() * sizeof(double)));
     cudaStream_t s = P->ctx->stream;
-    NM_TRY(copy_in(SG.pts.p, pts.data(), pts.size() * sizeof(double), s));
-    NM_TRY(copy_in(SG.invR.p, invR.data(), invR.size() * sizeof(double), s));
-    // the points in limbs, scaled by a power of two to [-1, 1]
+    // the points, scaled by a power of two to [-1, 1], and in limbs
     double far = 0;
     for (double v : pts) far = std::max(far, std::fabs(v));
     SG.inv_scale = far > 0 ? std::exp2(-std::ceil(std::log2(far))) : 1.0;
+    for (double& v : pts) v *= SG.inv_scale;
+    NM_TRY(copy_in(SG.pts.p, pts.data(), pts.size() * sizeof(double), s));
+    NM_TRY(copy_in(SG.invR.p, invR.data(), invR.size() * sizeof(double), s));
     NM_TRY(SG.cexp.alloc(64 * sizeof(int)));
     NM_TRY(SG.limbs.alloc(np * kLimbs * sizeof(float)));
-    split_points_kernel<<<1024, 256, 0, s>>>(np, 3, SG.pts.as<double>(), SG.inv_scale, SG.limbs.as<float>());
+    split_points_kernel<<<1024, 256, 0, s>>>(np, 3, SG.pts.as<double>(), 1.0, SG.limbs.as<float>());
     count_launch();
     NM_CUDA(cudaGetLastError());
     int* flag = SG.cexp.as<int>();   // free until the first product

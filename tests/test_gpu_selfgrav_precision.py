@@ -94,3 +94,32 @@ def test_error_of_the_term(case, problem, form, b):
     err = (got - ref).astype(float)
     rel = np.sqrt((err ** 2).mean() / (ref.astype(float) ** 2).mean())
     assert rel <= (4.6e-12 if form == "mixed" else 1.2e-12), rel
+
+
+@pytest.mark.parametrize("power", [70, -70])
+def test_double_form_in_any_units(power):
+    """Lengths in units of 2^power, G scaled so that every term of K_eff keeps
+    its share: the product is 2^power times that in plain units (a power of two
+    scales every step exactly; 1e-11 as for the product against the oracle).
+    Squared distances leave the float range."""
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_1906_11082_gb300 import nm
+    from synth.model import homogeneous_ball
+    out = []
+    for p in (0, power):
+        mesh, model = homogeneous_ball(h=0.45, seed=1)
+        mesh.xyz = mesh.xyz * 2.0 ** p
+        model.G = 2.0 ** (-2 * p) / np.pi
+        P = nm.Problem(nm.Context(0), mesh, model, self_gravity=True)
+        X = torch.randn((P.n, 5), dtype=torch.float64, device="cuda",
+                        generator=torch.Generator(device="cuda").manual_seed(2))
+        T, K = torch.empty_like(X), torch.empty_like(X)
+        P.apply_K(X, T)
+        nm.Problem(nm.Context(0), mesh, model).apply_K(X, K)
+        torch.cuda.synchronize()
+        out.append(((K - T) * 2.0 ** -p, K * 2.0 ** -p))
+    (t0, k0), (t1, k1) = out
+    assert float((k1 - k0).abs().max() / k0.abs().max()) <= 1e-11
+    assert float((t1 - t0).abs().max() / k0.abs().max()) <= 1e-11
+    assert float(t0.abs().max() / k0.abs().max()) > 1e-4   # the term counts
